@@ -311,6 +311,13 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
   return t;
 }
 
+// sqrt(sum b^2 / n) of the last completed iteration (0 before the first). Taken
+// once, with the outputs: an FP64 division and square root in every update
+// would add 0.4 us to each iteration.
+__device__ __forceinline__ double rms_residual(double sb2, int n) {
+  return n > 0 ? sqrt(sb2 / (double)n) : 0.0;
+}
+
 // The pair's state the solve reads, loaded by one thread at the start of the
 // epilogue (every load in flight at once, before the partials are combined)
 // instead of one after another at the end of the solve. The state was last
@@ -342,26 +349,157 @@ __device__ __forceinline__ PairPre load_pre(const PairState* st, int level) {
   return q;
 }
 
-// Eq. 5: (A^T A + 2 lambda n P^T P) x = A^T b, P = [I3 | 0]; Cholesky solve;
-// T <- [Exp(alpha, beta, gamma) | t] T; convergence control (Sec. 3.4).
-// FP64, run by one warp (the FP64 units are narrow on this part, so the
-// dependent chain, not the operation count, sets the time): a right-looking
-// Cholesky with one reciprocal square root per column and the trailing update
-// spread over lanes, substitutions by multiplication with the pivots'
-// inverses, and the pose composition and float32 transforms one entry per lane.
-// sm: >= 96 doubles of shared memory. Returns (in lane 0) the level the pair
-// iterates at next, or -1 when it has finished or stopped.
-// pre: the pair's state from load_pre, valid in lane 0.
+// 1 / d to the last bit or two: the hardware's reciprocal estimate r (20 bits
+// and more) and one third-order Householder step r (1 + e + e^2), e = 1 - d r,
+// whose error e^3 lies below an ulp. Three dependent FP64 operations where the
+// compiler's division takes twice the time.
+__device__ __forceinline__ double recip(double d) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+  const double e = fma(-d, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+__device__ __forceinline__ double lane_of(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
+
+// Lane of the upper-triangle entry (i, k), i <= k < 6, in the solve's layout.
+__device__ __forceinline__ int upper_lane(int i, int k) { return i * (11 - i) / 2 + k; }
+
+// Eq. 5: (A^T A + 2 lambda n P^T P) x = A^T b, P = [I3 | 0];
+// T <- [Exp(alpha, beta, gamma) | t] T, and the float32 transforms of the new
+// T. FP64, run by one warp, on values alone (S: the 29 sums in shared memory;
+// Tc: lane 4 i + j < 12 holds column j of T; Tmc: a lane o >= 12 holds the
+// column of Tm that its transform entry o needs, Tmt Tm's translation; gadd:
+// what lane 21 + r < 24 adds to its right-hand side).
+//
+// What bounds it is the chain of dependent FP64 operations (~64 cycles each on
+// this part), not their number, so the chain is kept short: lane (r, c) holds
+// one entry of the upper triangle, lane 21 + r the right-hand side, and step j
+// of a Gauss-Jordan elimination is one broadcast of the pivot, one reciprocal
+// and one fused multiply-add for all entries at once (the products H_rj H_jc
+// need no reciprocal and run beside it); eliminating above the pivot too
+// leaves no back substitution. A diagonal lane's last value is its pivot: the
+// system is degenerate when one is not above 1e-12 of its own entry of H.
+// Measured on GB300: 8.5 us for the Cholesky factorisation and substitutions
+// by one thread that this replaces, 3.9 us with this form (a 640x480 pair).
+struct Solved {
+  double x;     // lanes 21..26: the increment (alpha, beta, gamma, tx, ty, tz)
+  double T;     // lanes 0..11: the new pose, row-major
+  float xf;     // lanes 0..23: its float32 transforms (see xf_entry)
+  bool degenerate;
+};
+
+__device__ __forceinline__ Solved solve_lanes(const double* S, double reg, const double (&Tc)[3],
+                                              const double (&Tmc)[3], const double (&Tmt)[3],
+                                              double gadd) {
+  const int lane = threadIdx.x & 31;
+  const bool rhs = lane >= 21;
+  const int r = rhs ? min(lane - 21, 5)
+                    : (lane >= 6) + (lane >= 11) + (lane >= 15) + (lane >= 18) + (lane >= 20);
+  const int c = rhs ? 6 : lane - upper_lane(r, 0);
+  double h = S[min(lane, 26)] + (rhs ? gadd : (r == c && r < 3 ? reg : 0.0));
+  const double h0 = h;
+  double pinv = 0.0;
+#pragma unroll
+  for (int j = 0; j < 6; ++j) {
+    const double piv = lane_of(h, upper_lane(j, j));
+    const double a = lane_of(h, r > j ? upper_lane(j, r) : upper_lane(r, j));
+    const double b = lane_of(h, rhs ? 21 + j : upper_lane(j, max(c, j)));
+    const double ab = a * b;
+    const double ri = recip(piv);
+    if (r == j) pinv = ri;
+    else if (c > j) h = fma(-ab, ri, h);
+  }
+  Solved o;
+  o.degenerate = __any_sync(0xffffffffu, !rhs && r == c && !(h > 1e-12 * h0));
+  o.x = h * pinv;
+  const double w0 = lane_of(o.x, 21), w1 = lane_of(o.x, 22), w2 = lane_of(o.x, 23);
+  // Rodrigues: dR = I + A [w]x + B [w]x^2, A = sin(t)/t, B = (1 - cos t)/t^2;
+  // below t = 0.2 both from their Taylor series (truncation < 3e-15), A in the
+  // even lanes and B in the odd ones
+  const double th2 = fma(w2, w2, fma(w1, w1, w0 * w0));
+  double A, B;
+  if (th2 < 0.04) {
+    const bool odd = lane & 1;
+    double f = fma(th2, odd ? 1.0 / 3628800.0 : 1.0 / 362880.0, odd ? -1.0 / 40320.0 : -1.0 / 5040.0);
+    f = fma(th2, f, odd ? 1.0 / 720.0 : 1.0 / 120.0);
+    f = fma(th2, f, odd ? -1.0 / 24.0 : -1.0 / 6.0);
+    f = fma(th2, f, odd ? 0.5 : 1.0);
+    A = lane_of(f, 0);
+    B = lane_of(f, 1);
+  } else {
+    const double th = sqrt(th2);
+    double sn, cs;
+    sincos(th, &sn, &cs);
+    A = sn / th;
+    B = (1.0 - cs) / th2;
+  }
+  // lane 4 i + k: dR(i, k), with [w]x(i, k) = -+ the third component (+ where
+  // k is two after i) and [w]x^2 = w w^T - t^2 I; then lane 4 i + j: row i of
+  // dR times column j of T
+  const int i = min(lane >> 2, 2), j = lane & 3;
+  const double wi = i == 0 ? w0 : (i == 1 ? w1 : w2);
+  const double wk = j == 0 ? w0 : (j == 1 ? w1 : w2);
+  const int m = 3 - i - j;
+  const double wm = m == 0 ? w0 : (m == 1 ? w1 : w2);
+  const double K = i == j ? 0.0 : ((j - i + 3) % 3 == 2 ? wm : -wm);
+  const double dR = fma(B, fma(wi, wk, i == j ? -th2 : 0.0), fma(A, K, i == j ? 1.0 : 0.0));
+  double t = lane_of(o.x, 24 + i);
+  t = j == 3 ? t : 0.0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) t = fma(lane_of(dR, 4 * i + k), Tc[k], t);
+  o.T = t;
+  // entry o of the float32 transforms, operation for operation as xf_entry
+  const int q = max(lane - 12, 0);
+  const int ej = q < 9 ? q % 3 : 3;
+  const double rel = j == 3 ? __dsub_rn(t, i == 0 ? Tmt[0] : (i == 1 ? Tmt[1] : Tmt[2])) : t;
+  double s = __dmul_rn(Tmc[0], lane_of(rel, ej));
+  s = __dadd_rn(s, __dmul_rn(Tmc[1], lane_of(rel, 4 + ej)));
+  s = __dadd_rn(s, __dmul_rn(Tmc[2], lane_of(rel, 8 + ej)));
+  const double own = lane_of(t, lane < 9 ? (lane / 3) * 4 + lane % 3 : (lane < 12 ? (lane - 9) * 4 + 3 : 0));
+  o.xf = __double2float_rn(lane < 12 ? own : s);
+  return o;
+}
+
+// The column of Tm that transform entry `lane` needs, and Tm's translation.
+__device__ __forceinline__ void load_tm(const double* Tm, double (&Tmc)[3], double (&Tmt)[3]) {
+  const int q = max((int)(threadIdx.x & 31) - 12, 0);
+  const int ei = q < 9 ? q / 3 : min(q - 9, 2);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    Tmc[k] = Tm[4 * k + ei];
+    Tmt[k] = Tm[4 * k + 3];
+  }
+}
+
+// The prior-anchored variant's addition to the right-hand side, -2 lambda n r,
+// r = log(R R_prior^T), in lanes 21..23 (0 elsewhere): M = R R_prior^T one
+// entry per lane, then t = atan2(|v| / 2, (tr M - 1) / 2) and
+// r = t / (2 sin t) v, v = (M21 - M12, M02 - M20, M10 - M01).
+__device__ double anchored_rhs(const double* T, const double* prior_R, double reg) {
+  const int lane = threadIdx.x & 31;
+  double m = 0.0;
+  if (lane < 9)
+    for (int k = 0; k < 3; ++k) m += __ldcg(T + (lane / 3) * 4 + k) * __ldcg(prior_R + (lane % 3) * 3 + k);
+  const double v0 = lane_of(m, 7) - lane_of(m, 5), v1 = lane_of(m, 2) - lane_of(m, 6),
+               v2 = lane_of(m, 3) - lane_of(m, 1);
+  const double sn = 0.5 * sqrt(v0 * v0 + v1 * v1 + v2 * v2);
+  const double cs = 0.5 * (lane_of(m, 0) + lane_of(m, 4) + lane_of(m, 8) - 1.0);
+  const double t = atan2(sn, cs);
+  const double f = t < 1e-4 ? 0.5 * (1.0 + t * t / 6.0) : t / (2.0 * sn);
+  return lane == 21 ? -reg * f * v0 : lane == 22 ? -reg * f * v1 : lane == 23 ? -reg * f * v2 : 0.0;
+}
+
+// The solve and update of one pair (solve_lanes) and its bookkeeping:
+// convergence control (Sec. 3.4), the next iteration's window, the trace.
+// Run by one warp; pre: the pair's state from load_pre, valid in lane 0.
+// Returns (in lane 0) the level the pair iterates at next, or -1 when it has
+// finished or stopped.
 __device__ __noinline__ int solve_update_warp(const PairDesc* d, PairState* st, const double* S,
-                                               int level, const KParams& P, double* sm, int passes,
+                                               int level, const KParams& P, int passes,
                                                const PairPre& pre) {
   const int lane = threadIdx.x & 31;
   const unsigned long long t_start = globaltimer_ns();
-  double* H = sm;           // 36: H
-  double* g = sm + 42;      // 6: A^T b, then the increment x
-  double* Tn = sm + 54;     // 12: new pose
-  double* dR = sm + 66;     // 9
-  double* misc = sm + 75;   // [0] lambda [1] A [2] B
   const int n = (int)S[27];
   if (n < P.n_min) {
     if (lane == 0) {
@@ -370,140 +508,28 @@ __device__ __noinline__ int solve_update_warp(const PairDesc* d, PairState* st, 
     }
     return -1;
   }
-  if (lane == 0) misc[0] = lambda_of_n(P.lambda_mode, pre.lambda_c, n);
-  __syncwarp();
-  const double reg = (2.0 * misc[0]) * (double)n;
-  if (lane < 21) {  // upper-triangle sum `lane` -> (r, c)
-    int r = 0, k = lane;
-    while (k >= 6 - r) {
-      k -= 6 - r;
-      ++r;
-    }
-    const int c = r + k;
-    const double v = S[lane] + ((r == c && r < 3) ? reg : 0.0);
-    H[r * 6 + c] = v;
-    H[c * 6 + r] = v;
-  }
-  if (lane < 6) g[lane] = S[21 + lane];
-  __syncwarp();
-  if ((P.flags & KF_PRIOR_ANCHORED) && __shfl_sync(0xffffffffu, pre.has_prior, 0)) {
-    // prior-anchored variant: g_rot -= 2 lambda n r, r = log(R R_prior^T):
-    // M = R R_prior^T one entry per lane, then t = atan2(|v| / 2, (tr M - 1) / 2)
-    // and r = t / (2 sin t) v, v = (M21 - M12, M02 - M20, M10 - M01)
-    double* M = sm + 54;  // the new-pose scratch, free until the update
-    if (lane < 9) {
-      const int i = lane / 3, j = lane % 3;
-      double m = 0.0;
-      for (int k = 0; k < 3; ++k) m += __ldcg(&st->T[i * 4 + k]) * __ldcg(&st->prior_R[j * 3 + k]);
-      M[lane] = m;
-    }
-    __syncwarp();
-    if (lane == 0) {
-      const double v0 = M[7] - M[5], v1 = M[2] - M[6], v2 = M[3] - M[1];
-      const double sn = 0.5 * sqrt(v0 * v0 + v1 * v1 + v2 * v2);
-      const double cs = 0.5 * (M[0] + M[4] + M[8] - 1.0);
-      const double t = atan2(sn, cs);
-      const double f = t < 1e-4 ? 0.5 * (1.0 + t * t / 6.0) : t / (2.0 * sn);
-      g[0] -= reg * f * v0;
-      g[1] -= reg * f * v1;
-      g[2] -= reg * f * v2;
-    }
-    __syncwarp();
-  }
-  // Cholesky factorisation H = L L^T and the two triangular solves, by one
-  // thread in registers (the loops unroll to fixed indices): a chain of
-  // dependent FP64 operations costs ~64 cycles each here, and one thread
-  // avoids a warp barrier and a shared-memory round trip per step. A pivot
-  // not above 1e-12 of its own diagonal entry of H is degenerate.
-  int degenerate = 0;
-  if (lane == 0) {
-    double Lm[6][6], x[6];
+  double Tc[3], Tmc[3], Tmt[3];
 #pragma unroll
-    for (int i = 0; i < 6; ++i)
-#pragma unroll
-      for (int c = 0; c <= i; ++c) Lm[i][c] = H[i * 6 + c];
-#pragma unroll
-    for (int i = 0; i < 6; ++i) x[i] = g[i];
-    double r[6];
-#pragma unroll
-    for (int j = 0; j < 6; ++j) {
-      double a = Lm[j][j];
-#pragma unroll
-      for (int c = 0; c < j; ++c) a -= Lm[j][c] * Lm[j][c];
-      if (!(a > 1e-12 * H[j * 7])) degenerate = 1;
-      r[j] = rsqrt(a);
-      Lm[j][j] = a * r[j];
-#pragma unroll
-      for (int i = j + 1; i < 6; ++i) {
-        double v = Lm[i][j];
-#pragma unroll
-        for (int c = 0; c < j; ++c) v -= Lm[i][c] * Lm[j][c];
-        Lm[i][j] = v * r[j];
-      }
-    }
-#pragma unroll
-    for (int k = 0; k < 6; ++k) {  // L y = g
-      double v = x[k];
-#pragma unroll
-      for (int c = 0; c < k; ++c) v -= Lm[k][c] * x[c];
-      x[k] = v * r[k];
-    }
-#pragma unroll
-    for (int k = 5; k >= 0; --k) {  // L^T x = y
-      double v = x[k];
-#pragma unroll
-      for (int c = k + 1; c < 6; ++c) v -= Lm[c][k] * x[c];
-      x[k] = v * r[k];
-    }
-#pragma unroll
-    for (int i = 0; i < 6; ++i) g[i] = x[i];
-  }
-  degenerate = __shfl_sync(0xffffffffu, degenerate, 0);
-  if (degenerate) {
+  for (int k = 0; k < 3; ++k) Tc[k] = __ldcg(&st->T[4 * k + (lane & 3)]);
+  load_tm(d->Tm, Tmc, Tmt);
+  const double lam = lane_of(lane == 0 ? lambda_of_n(P.lambda_mode, pre.lambda_c, n) : 0.0, 0);
+  const double reg = (2.0 * lam) * (double)n;
+  double gadd = 0.0;
+  if ((P.flags & KF_PRIOR_ANCHORED) && __shfl_sync(0xffffffffu, pre.has_prior, 0))
+    gadd = anchored_rhs(st->T, st->prior_R, reg);
+  const Solved o = solve_lanes(S, reg, Tc, Tmc, Tmt, gadd);
+  if (o.degenerate) {
     if (lane == 0) {
       st->status = KF_ERR_DEGENERATE;
       st->stopped = 1;
     }
     return -1;
   }
-  __syncwarp();
-  // Rodrigues: dR = I + A [w]x + B [w]x^2, A = sin(t)/t, B = (1 - cos t)/t^2;
-  // below t = 0.2 both from their Taylor series (truncation < 3e-15)
-  if (lane == 0) {
-    const double th2 = g[0] * g[0] + g[1] * g[1] + g[2] * g[2];
-    if (th2 < 0.04) {
-      // multiplications by the coefficients' reciprocals (an FP64 division
-      // costs ~380 cycles here; the series is far from needing exact ones)
-      misc[1] = 1.0 - th2 * (1.0 / 6.0) * (1.0 - th2 * (1.0 / 20.0) * (1.0 - th2 * (1.0 / 42.0) * (1.0 - th2 * (1.0 / 72.0))));
-      misc[2] = 0.5 * (1.0 - th2 * (1.0 / 12.0) * (1.0 - th2 * (1.0 / 30.0) * (1.0 - th2 * (1.0 / 56.0) * (1.0 - th2 * (1.0 / 90.0)))));
-    } else {
-      const double th = sqrt(th2);
-      double sn, cs;
-      sincos(th, &sn, &cs);
-      misc[1] = sn / th;
-      misc[2] = (1.0 - cs) / th2;
-    }
-  }
-  __syncwarp();
-  if (lane < 9) {
-    const int i = lane / 3, j = lane % 3;
-    const double K[9] = {0.0, -g[2], g[1], g[2], 0.0, -g[0], -g[1], g[0], 0.0};
-    double k2 = 0.0;
-    for (int k = 0; k < 3; ++k) k2 += K[i * 3 + k] * K[k * 3 + j];
-    dR[lane] = (i == j ? 1.0 : 0.0) + misc[1] * K[lane] + misc[2] * k2;
-  }
-  __syncwarp();
-  if (lane < 12) {
-    const int i = lane / 4, j = lane % 4;
-    double v = 0.0;
-    for (int k = 0; k < 3; ++k) v += dR[i * 3 + k] * __ldcg(&st->T[k * 4 + j]);
-    if (j == 3) v += g[3 + i];
-    Tn[lane] = v;
-  }
-  __syncwarp();
-  if (lane < 12) st->T[lane] = Tn[lane];
-  if (lane < 24) st->xf[lane] = xf_entry(Tn, d->Tm, lane);
-  if (lane == 1) st->rms = sqrt(S[28] / (double)n);
+  if (lane < 12) st->T[lane] = o.T;
+  if (lane < 24) st->xf[lane] = o.xf;
+  double x[6];
+#pragma unroll
+  for (int i = 0; i < 6; ++i) x[i] = lane_of(o.x, 21 + i);
   if (lane != 0) return -1;
   // bookkeeping (the state's fields from pre)
   const int kmed = pre.kmed, N = pre.N, it = pre.it, tl = pre.tl;
@@ -521,8 +547,8 @@ __device__ __noinline__ int solve_update_warp(const PairDesc* d, PairState* st, 
     r.w0 = pre.w0;
     r.w1 = pre.w1;
     r.pad = 0;
-    r.lambda = misc[0];
-    for (int i = 0; i < 6; ++i) r.x[i] = g[i];
+    r.lambda = lam;
+    for (int i = 0; i < 6; ++i) r.x[i] = x[i];
     r.solve_ns = (int)(globaltimer_ns() - t_start);
   }
   st->iters[level] = it + 1;
@@ -530,6 +556,7 @@ __device__ __noinline__ int solve_update_warp(const PairDesc* d, PairState* st, 
   st->median_bin[level] = kmed;
   st->valid_pairs = N;
   st->inliers = n;
+  st->sb2 = S[28];
   int hl = pre.hl;
   int kh[kMaxWindow];
   for (int i = 0; i < kMaxWindow; ++i) kh[i] = pre.kh[i];
@@ -1105,14 +1132,13 @@ __device__ void reduce_items(const PairDesc* d, const LevelMaps& L, int first, i
 
 // The pair's reduction epilogue (block-wide, run by the block that finished
 // its last item): per sum, the items' partials in FP64 in a fixed order (slot
-// A + slot B on a hit, slot B alone otherwise; 8 strided sub-sums, then the 8
-// in order), the histogram cleared for the next iteration, then the solve and
+// A + slot B on a hit, slot B alone otherwise; 8 strided sub-sums, then a tree
+// over the 8), the histogram cleared for the next iteration, then the solve and
 // update (mode 2: the sums are stored instead). Returns (in thread 0) the
 // solve's next level (-1: finished or stopped).
 __device__ __noinline__ int combine_and_solve(const PairDesc* d, PairState* st, int count,
                                                int level, const KParams& P, int mode,
-                                               double (*s_part)[kSums], double* s_sums,
-                                               double* s_solve) {
+                                               double (*s_part)[kSums], double* s_sums) {
   __shared__ int s_hit;
   PairPre pre;
   if (threadIdx.x == 0) {
@@ -1127,8 +1153,8 @@ __device__ __noinline__ int combine_and_solve(const PairDesc* d, PairState* st, 
   const int hit = s_hit;
   // warp `sub` takes items sub, sub + 8, ...; lane k < 29 sums, per item, the
   // 16 rows of sum k (slot A's 8 warps, zero on a miss, and slot B's) in
-  // float32 by pairwise halving, then adds the items in increasing order in
-  // float64; four items' loads in flight. (The FP64 pipe of this part retires
+  // float32 by pairwise halving, then adds the items in float64, four at a
+  // time (their loads in flight together) as a tree, in increasing order. (The FP64 pipe of this part retires
   // about two additions per cycle per SM: a float64 chain over every row
   // would hold the pair's epilogue for microseconds.)
   const int k = threadIdx.x & 31, sub = threadIdx.x >> 5;
@@ -1152,10 +1178,7 @@ __device__ __noinline__ int combine_and_solve(const PairDesc* d, PairState* st, 
     for (; l + 24 < count; l += 32) {
       const float e0 = item_value(l), e1 = item_value(l + 8), e2 = item_value(l + 16),
                   e3 = item_value(l + 24);
-      t += (double)e0;
-      t += (double)e1;
-      t += (double)e2;
-      t += (double)e3;
+      t += ((double)e0 + (double)e1) + ((double)e2 + (double)e3);
     }
     for (; l < count; l += 8) t += (double)item_value(l);
   }
@@ -1163,9 +1186,14 @@ __device__ __noinline__ int combine_and_solve(const PairDesc* d, PairState* st, 
   for (int b = threadIdx.x; b < P.bins; b += kBlock) d->hist[b] = 0u;
   __syncthreads();
   if (threadIdx.x < kSums) {
-    double t = s_part[0][threadIdx.x];
-    for (int sub = 1; sub < 8; ++sub) t += s_part[sub][threadIdx.x];
-    s_sums[threadIdx.x] = t;
+    double v[kBlockWarps];
+#pragma unroll
+    for (int i = 0; i < kBlockWarps; ++i) v[i] = s_part[i][threadIdx.x];
+#pragma unroll
+    for (int h = 1; h < kBlockWarps; h <<= 1)
+#pragma unroll
+      for (int i = 0; i < kBlockWarps; i += 2 * h) v[i] += v[i + h];
+    s_sums[threadIdx.x] = v[0];
   }
   __syncthreads();
   int next = -1;
@@ -1174,7 +1202,7 @@ __device__ __noinline__ int combine_and_solve(const PairDesc* d, PairState* st, 
       if (threadIdx.x == 0)
         for (int k = 0; k < kSums; ++k) st->dbg_sums[k] = s_sums[k];
     } else {
-      next = solve_update_warp(d, st, s_sums, level, P, s_solve, hit ? 1 : 2, pre);
+      next = solve_update_warp(d, st, s_sums, level, P, hit ? 1 : 2, pre);
     }
     if (threadIdx.x == 0) d->counters[1] = 0u;
   }
@@ -1266,7 +1294,6 @@ __global__ void __launch_bounds__(kBlock, KF_REDUCE_MINB) k_reduce_solve(const P
   __shared__ int s_active, s_klo, s_khi, s_hit, s_last;
   __shared__ double s_sums[kSums];
   __shared__ double s_part[8][kSums];
-  __shared__ double s_solve[96];
   const int n_items = __ldcg(list);
   const int M = (n_items + gridDim.x - 1) / gridDim.x;
   int f = blockIdx.x * M;
@@ -1304,7 +1331,7 @@ __global__ void __launch_bounds__(kBlock, KF_REDUCE_MINB) k_reduce_solve(const P
       __syncthreads();
       if (s_last) {
         __threadfence();
-        combine_and_solve(d, st, count, level, P, mode, s_part, s_sums, s_solve);
+        combine_and_solve(d, st, count, level, P, mode, s_part, s_sums);
       }
     }
     f = run_end;
@@ -1354,7 +1381,7 @@ __device__ void init_state(const PairDesc* d, const PairInput& pi, const KParams
   st->w0 = st->w1 = -1;  // no band edge known yet: the first pass is histogram only
   st->hit = 0;
   st->valid_pairs = st->inliers = 0;
-  st->rms = 0.0;
+  st->sb2 = 0.0;
   st->trace_len = 0;
   d->counters[0] = 0u;
   d->counters[1] = 0u;
@@ -1392,7 +1419,7 @@ __global__ void k_icp_finish(const PairDesc* const* descs, PairOutput* out) {
   o.res.total_iters = st->total_iters;
   o.res.inliers = st->inliers;
   o.res.valid_pairs = st->valid_pairs;
-  o.res.rms_residual = st->rms;
+  o.res.rms_residual = rms_residual(st->sb2, st->inliers);
 }
 
 __global__ void __launch_bounds__(kBlock) k_debug_setup(const PairDesc* const* self,
@@ -1577,7 +1604,7 @@ __device__ void finish_pair(const PairDesc* d, PairOutput* o, int n, unsigned* q
     o->res.total_iters = __ldcg(&st->total_iters);
     o->res.inliers = __ldcg(&st->inliers);
     o->res.valid_pairs = __ldcg(&st->valid_pairs);
-    o->res.rms_residual = __ldcg(&st->rms);
+    o->res.rms_residual = rms_residual(__ldcg(&st->sb2), __ldcg(&st->inliers));
   }
   __threadfence();
   __syncthreads();
@@ -1601,7 +1628,7 @@ __global__ void __launch_bounds__(kBlock, KF_SCHED_MINB) k_icp_sched(const PairD
   __shared__ int s_last, s_flag, s_a, s_b, s_hit;
   __shared__ double s_sums[kSums];
   __shared__ double s_part[8][kSums];
-  __shared__ double s_solve[96];
+  __shared__ double s_seed[12];
   // seed: every block that starts takes unseeded pairs until none is left
   for (;;) {
     if (threadIdx.x == 0) s_word = atomicAdd(qh + kQSeed, 1u);
@@ -1610,7 +1637,7 @@ __global__ void __launch_bounds__(kBlock, KF_SCHED_MINB) k_icp_sched(const PairD
     __syncthreads();
     if (p >= (unsigned)n) break;
     const PairDesc* d = descs[p];
-    seed_pair(d, in[p], P, s_solve);
+    seed_pair(d, in[p], P, s_seed);
     const int level = P.levels - 1;
     push_stage(qh, qs, qmask, n, (int)p, level, 0, items_of(d, level));
   }
@@ -1675,7 +1702,7 @@ __global__ void __launch_bounds__(kBlock, KF_SCHED_MINB) k_icp_sched(const PairD
         } else if (s_hit) {
           fixup_all(d, count, chunk, s_a, s_b);
           __threadfence();
-          const int next = combine_and_solve(d, st, count, level, P, 0, s_part, s_sums, s_solve);
+          const int next = combine_and_solve(d, st, count, level, P, 0, s_part, s_sums);
           if (threadIdx.x == 0) s_flag = next;
           __syncthreads();
           const int nl = s_flag;
@@ -1707,7 +1734,7 @@ __global__ void __launch_bounds__(kBlock, KF_SCHED_MINB) k_icp_sched(const PairD
       __syncthreads();
       if (s_last) {
         __threadfence();
-        const int next = combine_and_solve(d, st, count, level, P, 0, s_part, s_sums, s_solve);
+        const int next = combine_and_solve(d, st, count, level, P, 0, s_part, s_sums);
         if (threadIdx.x == 0) s_flag = next;
         __syncthreads();
         const int nl = s_flag;

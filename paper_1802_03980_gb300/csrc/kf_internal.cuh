@@ -89,7 +89,7 @@ struct PairState {
   int hit;                    // 1: the band edge fell in the window, the
                               // reduction pass adds the recorded pixels only
   int valid_pairs, inliers;   // last completed iteration
-  double rms;
+  double sb2;                 // sum b^2 over its inliers
   double dbg_sums[kSums];     // filled by the reduction stage in inspection mode
   double prior_R[9];          // IMU prior rotation (valid when has_prior)
   int has_prior;
