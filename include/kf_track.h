@@ -299,7 +299,9 @@ kf_status kf_debug_trace(kf_tracker* t, kf_iter_record* rec, int max, int* count
  * over an empty batch with every wait limited to wait_ms (clamped to 1..2000):
  * no task is ever queued, so each block's wait for its next task runs out,
  * sets the launch's error word and returns, and the call reports that as a
- * normal status. Returns KF_ERR_TIMEOUT when the error word was set (the
+ * normal status. With a frame and a model set, the launch that small batches
+ * take is checked too, its leader block alone: the counts it waits for never
+ * come. Returns KF_ERR_TIMEOUT when the error word was set (the
  * expected outcome), KF_ERR_INTERNAL if the launch ended without it, or a CUDA
  * error. The tracker stays usable; its frame, model and plans are untouched. */
 kf_status kf_debug_wait_timeout(kf_tracker* t, double wait_ms);

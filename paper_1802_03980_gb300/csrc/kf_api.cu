@@ -34,6 +34,8 @@ struct Plan {
   unsigned qmask = 0;                    // slots - 1 (a power of two)
   int grid = 0;                          // blocks of the scheduled launch
   bool sched = false;                    // one persistent launch (else per-iteration launches)
+  bool team = false;                     // one cooperative launch, a team of blocks per pair
+  TeamArgs args = {};                    // of the team launch
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   bool profiled = false;
@@ -83,6 +85,11 @@ struct kf_tracker {
   int* d_dbg_list = nullptr;
   unsigned* d_dbg_counter = nullptr;
   double* d_dbg_pose = nullptr;
+  void* d_team = nullptr;           // the team launch's buffers (see PairDesc)
+  size_t team_bytes = 0;
+  unsigned team_epoch = 0;          // team launches since the buffers were zeroed
+  bool team_dirty = false;          // a launch ended early: zero them first
+  int team_blocks = 0;              // blocks of a team launch that can be resident
   int max_items = 0;
   int grid_assoc = 0, grid_reduce = 0, grid_sched = 0;
   bool has_frame = false, has_model = false;
@@ -149,7 +156,9 @@ KParams make_kparams(const kf_params* p) {
   k.bins = p->hist_bins;
   k.d_max32 = (float)p->d_max;
   k.scale32 = (float)((double)p->hist_bins / p->d_max);
+  k.tiny_bins = !(k.d_max32 > 0x1p-49f && k.scale32 < 0x1p49f);
   k.kappa = p->band_kappa;
+  k.kappa_one = p->band_kappa == 1.0;
   k.cos_min32 = (float)p->cos_angle_min;
   k.use_angle = p->cos_angle_min > -1.0;
   k.conv_window = p->conv_window;
@@ -294,6 +303,64 @@ kf_status frame_stage(kf_tracker* t, size_t bytes) {
   return KF_OK;
 }
 
+// The team launch's blocks: per pair a leader and workers of at most
+// kTeamSlots half items each; false when the pairs do not fit the device.
+bool plan_teams(kf_tracker* const* trk, Plan* pl) {
+  const kf_tracker* t0 = trk[0];
+  const int n = pl->n;
+  if ((t0->kp.flags & KF_LAUNCH_PER_ITERATION) || n > kTeamMaxPairs || t0->team_blocks <= n) return false;
+  long long total = 0;
+  int halves[kTeamMaxPairs];
+  for (int k = 0; k < n; ++k) {
+    const kf_tracker* t = trk[pl->order[k]];
+    if (!t->d_team) return false;
+    const long long px = (long long)t->h_desc.lv[0].fw * t->h_desc.lv[0].fh;
+    halves[k] = 2 * (int)((px + level_chunk(0) - 1) / level_chunk(0));  // the widest level
+    total += halves[k];
+  }
+  const long long room = t0->team_blocks - n;
+  pl->grid = 0;
+  for (int k = 0; k < n; ++k) {
+    const long long most = std::min((long long)halves[k], std::max(1LL, room * halves[k] / total));
+    const int slots = (int)((halves[k] + most - 1) / most);
+    if (slots > kTeamSlots) return false;
+    TeamPair& tp = pl->args.pair[k];
+    tp.d = trk[pl->order[k]]->d_desc;
+    tp.first = pl->grid;
+    tp.workers = (halves[k] + slots - 1) / slots;
+    pl->grid += 1 + tp.workers;
+  }
+  pl->args.n = n;
+  pl->args.limit_ns = kSchedWaitLimitNs;
+  return pl->grid <= t0->team_blocks;
+}
+
+// Queues the team launch of a plan whose inputs are in h_in.
+kf_status launch_teams(kf_tracker* const* trk, Plan* pl, cudaStream_t s) {
+  kf_tracker* t0 = trk[0];
+  for (int k = 0; k < pl->n; ++k) {
+    kf_tracker* t = trk[pl->order[k]];
+    // a tag repeats after 2^20 launches: start again from zeroed buffers then,
+    // and after a launch that ended before its last clear
+    if (t->team_dirty || (t->team_epoch + 1) * (unsigned long long)kTeamTags >= (1ull << 32)) {
+      KF_CK(t0, cudaMemsetAsync(t->d_team, 0, t->team_bytes, s));
+      t->team_epoch = 0;
+    }
+    t->team_dirty = true;  // until the outputs say otherwise
+    pl->args.pair[k].tag = ++t->team_epoch * kTeamTags;
+    pl->args.pair[k].out = pl->h_out + k;
+    pl->args.in[k] = pl->h_in[k];
+    pl->h_out[k].res.status = KF_ERR_TIMEOUT;
+  }
+  if (pl->profiled) {
+    KF_CK(t0, cudaEventRecord(pl->ev[0], s));
+    KF_CK(t0, cudaEventRecord(pl->ev[1], s));
+  }
+  KF_CK(t0, launch_icp_team(pl->args, pl->grid, t0->kp, s));
+  if (pl->profiled) KF_CK(t0, cudaEventRecord(pl->ev[2], s));
+  return KF_OK;
+}
+
 kf_status build_plan(kf_tracker* const* trk, int n, Plan** slot) {
   kf_tracker* t0 = trk[0];
   plan_free(*slot);
@@ -309,6 +376,29 @@ kf_status build_plan(kf_tracker* const* trk, int n, Plan** slot) {
   for (int i = 0; i < n; ++i) pl->order[i] = i;
   auto px0 = [&](int i) { return (long long)trk[i]->h_desc.lv[0].fw * trk[i]->h_desc.lv[0].fh; };
   std::stable_sort(pl->order.begin(), pl->order.end(), [&](int a, int b) { return px0(a) > px0(b); });
+  pl->team = plan_teams(trk, pl);
+  if (pl->team) {
+    cudaError_t e = cudaMallocHost(&pl->h_in, sizeof(PairInput) * n);
+    if (e == cudaSuccess) e = cudaMallocHost(&pl->h_out, sizeof(PairOutput) * n);
+    pl->profiled = t0->profiling;
+    if (pl->profiled) {
+      pl->ev.resize(3, nullptr);
+      pl->ev_kind = {-1, 3, -1};
+      for (auto& ev : pl->ev)
+        if (e == cudaSuccess) e = cudaEventCreate(&ev);
+      for (int k = 0; k < n; ++k)
+        for (int l = 0; l < t0->p.levels; ++l) {
+          const LevelMaps& L = trk[pl->order[k]]->h_desc.lv[l];
+          pl->pair_px.push_back((long long)L.fw * L.fh);
+        }
+    }
+    if (e != cudaSuccess) {
+      plan_free(pl);
+      return cuda_fail(t0, e, "building the alignment plan");
+    }
+    *slot = pl;
+    return KF_OK;
+  }
   std::vector<const PairDesc*> descs(n);
   for (int k = 0; k < n; ++k) descs[k] = trk[pl->order[k]]->d_desc;
   const int L = t0->p.levels;
@@ -565,6 +655,19 @@ kf_status kf_track_create(const kf_params* p, int max_w, int max_h, void* cuda_s
   if ((e = tmalloc(t, &D.recs, 2 * sizeof(float4) * (px0 + kChunk))) != cudaSuccess) return bail(e);
   if ((e = tmalloc(t, &D.wcount, sizeof(unsigned) * kBlockWarps * t->max_items)) != cudaSuccess)
     return bail(e);
+  if (t->max_items <= kTeamMaxItems) {
+    const size_t hist = sizeof(unsigned) * 3 * team_hist_words(p->hist_bins);
+    const size_t msg = (hist + 255) / 256 * 256, rows = msg + 32 * sizeof(unsigned long long);
+    t->team_bytes = rows + (size_t)t->max_items * 2 * 32 * sizeof(unsigned long long);
+    char* area = nullptr;
+    if ((e = tmalloc(t, &area, t->team_bytes)) != cudaSuccess) return bail(e);
+    if ((e = cudaMemsetAsync(area, 0, t->team_bytes, t->stream)) != cudaSuccess) return bail(e);
+    t->d_team = area;
+    D.team_hist = reinterpret_cast<unsigned*>(area);
+    D.team_msg = reinterpret_cast<unsigned long long*>(area + msg);
+    D.team_rows = reinterpret_cast<unsigned long long*>(area + rows);
+    t->team_blocks = team_blocks(t->kp);
+  }
   if ((e = tmalloc(t, &t->d_desc, sizeof(PairDesc))) != cudaSuccess) return bail(e);
   if ((e = tmalloc(t, &t->d_self, sizeof(PairDesc*))) != cudaSuccess) return bail(e);
   if ((e = tmalloc(t, &t->d_dbg_list, sizeof(int) * list_ints(1))) != cudaSuccess) return bail(e);
@@ -826,11 +929,25 @@ kf_status kf_align_batch(kf_tracker* const* trk, int n, const double* prior_R,
       in.lambda = lambda[i] < 0 ? t0->p.lambda_c : lambda[i];
       in.has_prior = prior_R ? 1 : 0;
     }
-    KF_CK(t0, cudaMemcpyAsync(pl->d_in, pl->h_in, sizeof(PairInput) * n, cudaMemcpyHostToDevice, s));
-    KF_CK(t0, cudaGraphLaunch(pl->exec, s));
-    // outputs and, after them, the scheduled launch's queue header (error word)
-    KF_CK(t0, cudaMemcpyAsync(pl->h_out, pl->d_out, pl->out_pad + 512, cudaMemcpyDeviceToHost, s));
-    KF_CK(t0, cudaStreamSynchronize(s));
+    if (pl->team) {
+      // inputs in the launch's parameters, outputs written to pinned host memory
+      kf_status st = launch_teams(trk, pl, s);
+      if (st != KF_OK) return st;
+      KF_CK(t0, cudaStreamSynchronize(s));
+      for (int k = 0; k < n; ++k) {
+        const int st = pl->h_out[k].res.status;
+        if (st == KF_ERR_TIMEOUT)
+          return fail(t0, KF_ERR_TIMEOUT, "a bounded device wait of the team ICP launch ran out");
+        // too few matches ends a pair before its last histogram is cleared
+        trk[pl->order[k]]->team_dirty = st == KF_ERR_TOO_FEW_INLIERS;
+      }
+    } else {
+      KF_CK(t0, cudaMemcpyAsync(pl->d_in, pl->h_in, sizeof(PairInput) * n, cudaMemcpyHostToDevice, s));
+      KF_CK(t0, cudaGraphLaunch(pl->exec, s));
+      // outputs and, after them, the scheduled launch's queue header (error word)
+      KF_CK(t0, cudaMemcpyAsync(pl->h_out, pl->d_out, pl->out_pad + 512, cudaMemcpyDeviceToHost, s));
+      KF_CK(t0, cudaStreamSynchronize(s));
+    }
     if (pl->sched) {
       const unsigned* qh = reinterpret_cast<const unsigned*>(reinterpret_cast<const char*>(pl->h_out) + pl->out_pad);
       if (qh[kQErr] != 0u)
@@ -1050,6 +1167,25 @@ kf_status kf_debug_wait_timeout(kf_tracker* t, double wait_ms) {
     cudaFree(queue);
     if (e != cudaSuccess) return cuda_fail(t, e, "kf_debug_wait_timeout");
     if (err == 0u) return fail(t, KF_ERR_INTERNAL, "the empty scheduled launch ended without a wait running out");
+    // and a team's leader without its workers: the frame's pixels never arrive
+    if (t->d_team && t->has_frame && t->has_model) {
+      TeamArgs args = {};
+      PairOutput* out = nullptr;
+      KF_CK(t, cudaMallocHost(&out, sizeof(PairOutput)));
+      out->res.status = KF_ERR_TIMEOUT;
+      args.pair[0].d = t->d_desc;
+      args.pair[0].out = out;
+      args.pair[0].tag = ++t->team_epoch * kTeamTags;
+      args.n = 1;
+      args.limit_ns = (unsigned long long)(ms * 1e6);
+      t->team_dirty = true;
+      e = launch_icp_team(args, 1, t->kp, s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      const int st = out->res.status;
+      cudaFreeHost(out);
+      if (e != cudaSuccess) return cuda_fail(t, e, "kf_debug_wait_timeout");
+      if (st != KF_ERR_TIMEOUT) return fail(t, KF_ERR_INTERNAL, "a leader without workers ended without its wait running out");
+    }
     return fail(t, KF_ERR_TIMEOUT, "a bounded device wait ran out (expected: nothing was queued)");
   } catch (...) {
     return KF_ERR_INTERNAL;

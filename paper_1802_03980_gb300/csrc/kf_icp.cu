@@ -14,34 +14,17 @@
 // epilogue (median and band after the histogram; solve and update after the
 // reduction) runs in the pair's last block to finish, found with a per-pair
 // arrival counter (no block ever waits for another).
-#include "kf_internal.cuh"
+#include "kf_icp.cuh"
 
-// Tuning of the ICP kernels: minimum resident blocks per SM (register cap)
-// and frame pixels per thread per batch of the association passes.
+// Tuning of the ICP kernels: minimum resident blocks per SM (register cap).
 #ifndef KF_ASSOC_MINB
 #define KF_ASSOC_MINB 2
-#endif
-#ifndef KF_ASSOC_U
-#define KF_ASSOC_U 4
 #endif
 #ifndef KF_REDUCE_MINB
 #define KF_REDUCE_MINB 2
 #endif
 #ifndef KF_SCHED_MINB
 #define KF_SCHED_MINB 2
-#endif
-// Prefetch during an association batch: 0 none; 1 the warp's frame-vertex
-// lines of its next batch into L2; 2 also the model lines its next batch is
-// likely to gather (the warp's current match offset applied to the next
-// pixels); 3 and 4 as 1 and 2, into L1
-#ifndef KF_PREFETCH
-#define KF_PREFETCH 1
-#endif
-// Per-thread sums: 0 plain float32 fused multiply-adds; 1 compensated
-// (Kahan) summation, each sum carrying its lost low-order part in a second
-// register (a measurement build: twice the sum registers)
-#ifndef KF_KAHAN
-#define KF_KAHAN 0
 #endif
 // Scheduled kernel: the pair's median epilogue also runs the reduction pass
 // of a hit while the pairs still running number at least the launch's
@@ -54,168 +37,16 @@
 namespace kf {
 
 #ifdef KF_CHECKED
-__device__ long long g_fault[3];
-__device__ void kf_fault(int code, long long a, long long b) {
-  if (atomicCAS(reinterpret_cast<unsigned long long*>(&g_fault[0]), 0ull, (unsigned long long)code) == 0ull) {
-    g_fault[1] = a;
-    g_fault[2] = b;
-  }
-}
 void checked_fault(long long out[3]) {
-  cudaMemcpyFromSymbol(out, g_fault, sizeof(long long) * 3);
-  const long long z[3] = {0, 0, 0};
-  cudaMemcpyToSymbol(g_fault, z, sizeof(z));
+  out[0] = out[1] = out[2] = 0;
+  take_fault(out);
+  checked_fault_team(out);
 }
 #else
 void checked_fault(long long out[3]) { out[0] = out[1] = out[2] = 0; }
 #endif
 
 namespace {
-
-// ---------------------------------------------------------------------------
-// float32 decision chain. Every operation is one explicitly rounded IEEE
-// operation in a fixed order (a fused multiply-add where fmaf is written, no
-// other contraction), so that a float32 re-evaluation elsewhere reproduces
-// each decision bit for bit:
-//   row(R, t, v) = fma(R2, v.z, fma(R1, v.y, fma(R0, v.x, t)))
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ float row3(const float* R, float t, float x, float y, float z) {
-  return fmaf(R[2], z, fmaf(R[1], y, fmaf(R[0], x, t)));
-}
-
-__device__ __forceinline__ float rot3(const float* R, float x, float y, float z) {
-  return fmaf(R[2], z, fmaf(R[1], y, fmaf(R[0], x, 0.f)));
-}
-
-// Projective association (Sec. 3.2), split in two phases so that a thread
-// can issue the model gathers of several pixels before using any of them.
-//
-// project(): frame vertex v -> model pixel index j (or -1) and world point p.
-//   model-camera point m = T_rel v; reject unless m.z > 0;
-//   (u, v)^ = rint(fma(f m.xy, 1 / m.z, c)), round half to even; reject
-//   outside the image.
-// bin_of(): with the gathered model vertex q, d = |p - q| (point-to-point);
-//   reject unless d < d_max (NaN model holes fail too); bin = floor(d B / d_max).
-// xf: Rw[9] tw[3] (camera -> world) Rr[9] tr[3] (camera -> model camera).
-__device__ __forceinline__ int project(const LevelMaps& L, float vx, float vy, float vz,
-                                       const float* xf, float* p) {
-  const float mx = row3(xf + 12, xf[21], vx, vy, vz);
-  const float my = row3(xf + 15, xf[22], vx, vy, vz);
-  const float mz = row3(xf + 18, xf[23], vx, vy, vz);
-  p[0] = row3(xf + 0, xf[9], vx, vy, vz);
-  p[1] = row3(xf + 3, xf[10], vx, vy, vz);
-  p[2] = row3(xf + 6, xf[11], vx, vy, vz);
-  if (!(mz > 0.f)) return -1;  // also rejects invalid (NaN) frame vertices
-  const float rz = __frcp_rn(mz);  // 1 / m.z, rounded once
-  const float uf = fmaf(__fmul_rn(L.mfx, mx), rz, L.mcx);
-  const float vf = fmaf(__fmul_rn(L.mfy, my), rz, L.mcy);
-  const float ur = rintf(uf), vr = rintf(vf);
-  if (!(ur >= 0.f && ur <= (float)(L.mw - 1) && vr >= 0.f && vr <= (float)(L.mh - 1))) return -1;
-  return (int)vr * L.mw + (int)ur;
-}
-
-__device__ __forceinline__ int bin_of(const float* p, const float* q, const KParams& P) {
-  const float dx = __fsub_rn(p[0], q[0]);
-  const float dy = __fsub_rn(p[1], q[1]);
-  const float dz = __fsub_rn(p[2], q[2]);
-  const float d2 = fmaf(dz, dz, fmaf(dy, dy, __fmul_rn(dx, dx)));
-  const float d = __fsqrt_rn(d2);
-  if (!(d < P.d_max32)) return -1;
-  const int k = (int)floorf(__fmul_rn(d, P.scale32));
-  return k < P.bins - 1 ? k : P.bins - 1;
-}
-
-// Optional normal-angle gate: (R_cur n_frame) . n_model >= cos_min, float32.
-__device__ __forceinline__ bool angle_ok(const float* xf, const float* nf, const float* nq,
-                                         const KParams& P) {
-  const float wx = rot3(xf + 0, nf[0], nf[1], nf[2]);
-  const float wy = rot3(xf + 3, nf[0], nf[1], nf[2]);
-  const float wz = rot3(xf + 6, nf[0], nf[1], nf[2]);
-  float dot = __fadd_rn(__fmul_rn(wx, nq[0]), __fmul_rn(wy, nq[1]));
-  dot = __fadd_rn(dot, __fmul_rn(wz, nq[2]));
-  return dot >= P.cos_min32;
-}
-
-// Association variants (template bits): kAGate = the normal-angle gate,
-// kAShoot = normal shooting instead of the projected pixel.
-constexpr int kAGate = 1, kAShoot = 2;
-
-// Normal shooting (Sec. 3.3): among the valid model pixels of the
-// (2w+1)^2 window around the projected pixel jc, the one whose vertex q lies
-// closest to the line through the world point p along the world frame normal
-// n. Squared distance to the line, float32, each operation rounded in this
-// order: e = q - p; s = (e.x n.x + e.y n.y) + e.z n.z;
-// l2 = ((e.x^2 + e.y^2) + e.z^2) - s s. Candidates row by row, a strictly
-// smaller l2 replaces the best (ties keep the first). Holes (NaN vertex)
-// are skipped. Returns the chosen pixel (or -1) and its vertex in q.
-template <class T>
-__device__ __forceinline__ int shoot(const LevelMaps& L, const T* mV, int jc, const float* p,
-                                     const float* n, int w, float* q) {
-  constexpr int kRow = 9;  // 2 w + 1 for the largest window (w = 4)
-  const int mn = L.mw * L.mh;
-  const int cu = jc % L.mw, cv = jc / L.mw;
-  const float nan = __int_as_float(0x7fc00000);
-  float best = __int_as_float(0x7f800000);
-  int bj = -1;
-  for (int dy = -w; dy <= w; ++dy) {
-    const int y = cv + dy;
-    if (y < 0 || y >= L.mh) continue;
-    // one row of candidates loaded together, then compared in order
-    float cx[kRow], cy[kRow], cz[kRow];
-#pragma unroll
-    for (int k = 0; k < kRow; ++k) {
-      const int x = cu - w + k;
-      const bool in = k <= 2 * w && x >= 0 && x < L.mw;
-      const int j = y * L.mw + (in ? x : cu);
-      cx[k] = in ? Store<T>::ld(mV, j) : nan;
-      cy[k] = in ? Store<T>::ld(mV, mn + j) : nan;
-      cz[k] = in ? Store<T>::ld(mV, 2 * mn + j) : nan;
-    }
-#pragma unroll
-    for (int k = 0; k < kRow; ++k) {
-      if (isnan(cx[k])) continue;  // outside the window or the image, or a hole
-      const float ex = __fsub_rn(cx[k], p[0]), ey = __fsub_rn(cy[k], p[1]), ez = __fsub_rn(cz[k], p[2]);
-      float sd = __fadd_rn(__fmul_rn(ex, n[0]), __fmul_rn(ey, n[1]));
-      sd = __fadd_rn(sd, __fmul_rn(ez, n[2]));
-      float ee = __fadd_rn(__fmul_rn(ex, ex), __fmul_rn(ey, ey));
-      ee = __fadd_rn(ee, __fmul_rn(ez, ez));
-      const float l2 = __fsub_rn(ee, __fmul_rn(sd, sd));
-      if (l2 < best) {
-        best = l2;
-        bj = y * L.mw + cu - w + k;
-        q[0] = cx[k];
-        q[1] = cy[k];
-        q[2] = cz[k];
-      }
-    }
-  }
-  return bj;
-}
-
-// Entry o (0..23) of the float32 transforms: Rw[9] tw[3] are T_cur rounded to
-// float32; Rr[9] tr[3] are the FP64 relative transform T_m^-1 T_cur, summed
-// in the order k = 0, 1, 2 with explicitly rounded operations, then rounded.
-__device__ __forceinline__ float xf_entry(const double* T, const double* Tm, int o) {
-  if (o < 9) return __double2float_rn(T[(o / 3) * 4 + o % 3]);
-  if (o < 12) return __double2float_rn(T[(o - 9) * 4 + 3]);
-  if (o < 21) {
-    const int i = (o - 12) / 3, j = (o - 12) % 3;
-    double s = __dmul_rn(Tm[0 * 4 + i], T[0 * 4 + j]);
-    s = __dadd_rn(s, __dmul_rn(Tm[1 * 4 + i], T[1 * 4 + j]));
-    s = __dadd_rn(s, __dmul_rn(Tm[2 * 4 + i], T[2 * 4 + j]));
-    return __double2float_rn(s);
-  }
-  const int i = o - 21;
-  const double d0 = __dsub_rn(T[3], Tm[3]), d1 = __dsub_rn(T[7], Tm[7]), d2 = __dsub_rn(T[11], Tm[11]);
-  double s = __dmul_rn(Tm[0 * 4 + i], d0);
-  s = __dadd_rn(s, __dmul_rn(Tm[1 * 4 + i], d1));
-  s = __dadd_rn(s, __dmul_rn(Tm[2 * 4 + i], d2));
-  return __double2float_rn(s);
-}
-
-__device__ void compute_xf(const double* T, const double* Tm, float* xf) {
-  for (int o = 0; o < 24; ++o) xf[o] = xf_entry(T, Tm, o);
-}
 
 // Median bin k_med = min{k : 2 C(k) >= N} from the pair's histogram and the
 // band of bins around it (Sec. 3.3). Block-wide; the caller is the pair's last
@@ -276,333 +107,29 @@ __device__ __noinline__ int median_and_band(const PairDesc* d, PairState* st, co
       st->stopped = 1;
       stop = 1;
     }
-    int klo = 0, khi = B - 1;
-    if (P.flags & KF_USE_FILTER) {
-      const double m = (double)kmed + 0.5;
-      khi = (int)floor(__dmul_rn(__dadd_rn(1.0, P.kappa), m));
-      klo = (int)ceil(__dmul_rn(__dsub_rn(1.0, P.kappa), m)) - 1;
-      khi = khi < B - 1 ? khi : B - 1;
-      klo = klo > 0 ? klo : 0;
-    }
+    int klo, khi;
+    band_of(P, kmed, klo, khi);
     st->klo = klo;
     st->khi = khi;
-    // the association pass summed bins < w0 and recorded bins [w0, w1): the
-    // band [0, khi] is complete from those when khi lies in [w0 - 1, w1 - 1]
-    const int w0 = __ldcg(&st->w0), w1 = __ldcg(&st->w1);
-    st->hit = (w0 >= 0 && klo == 0 && khi >= w0 - 1 && khi <= w1 - 1) ? 1 : 0;
+    st->hit = band_hits(klo, khi, __ldcg(&st->w0), __ldcg(&st->w1)) ? 1 : 0;
   }
   return stop;
 }
 
-__device__ double lambda_of_n(int mode, double c, int n) {
-  const double dn = (double)n;
-  switch (mode) {
-    case KF_LAMBDA_C_SQRT_N: return c / sqrt(dn);
-    case KF_LAMBDA_C_N: return c / dn;
-    case KF_LAMBDA_C_N2: return c / (dn * dn);
-    case KF_LAMBDA_C_LOG_N: return c * log(dn);
-    default: return c;
-  }
-}
-
-__device__ __forceinline__ unsigned long long globaltimer_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-  return t;
-}
-
-// sqrt(sum b^2 / n) of the last completed iteration (0 before the first). Taken
-// once, with the outputs: an FP64 division and square root in every update
-// would add 0.4 us to each iteration.
-__device__ __forceinline__ double rms_residual(double sb2, int n) {
-  return n > 0 ? sqrt(sb2 / (double)n) : 0.0;
-}
-
-// The pair's state the solve reads, loaded by one thread at the start of the
-// epilogue (every load in flight at once, before the partials are combined)
-// instead of one after another at the end of the solve. The state was last
-// written by other blocks (the histogram epilogue, earlier solves): every
-// read goes through L2.
-struct PairPre {
-  double lambda_c;
-  int kmed, N, klo, khi, w0, w1, it, tl, total, hl, status, has_prior;
-  int kh[kMaxWindow];
-};
-
-__device__ __forceinline__ PairPre load_pre(const PairState* st, int level) {
-  PairPre q;
-  q.lambda_c = __ldcg(&st->lambda_c);
-  q.kmed = __ldcg(&st->kmed);
-  q.N = __ldcg(&st->N);
-  q.klo = __ldcg(&st->klo);
-  q.khi = __ldcg(&st->khi);
-  q.w0 = __ldcg(&st->w0);
-  q.w1 = __ldcg(&st->w1);
-  q.it = __ldcg(&st->iters[level]);
-  q.tl = __ldcg(&st->trace_len);
-  q.total = __ldcg(&st->total_iters);
-  q.hl = __ldcg(&st->hist_len);
-  q.status = __ldcg(&st->status);
-  q.has_prior = __ldcg(&st->has_prior);
-#pragma unroll
-  for (int i = 0; i < kMaxWindow; ++i) q.kh[i] = __ldcg(&st->kmed_hist[i]);
-  return q;
-}
-
-// 1 / d to the last bit or two: the hardware's reciprocal estimate r (20 bits
-// and more) and one third-order Householder step r (1 + e + e^2), e = 1 - d r,
-// whose error e^3 lies below an ulp. Three dependent FP64 operations where the
-// compiler's division takes twice the time.
-__device__ __forceinline__ double recip(double d) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
-  const double e = fma(-d, r, 1.0);
-  return fma(r, fma(e, e, e), r);
-}
-
-__device__ __forceinline__ double lane_of(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
-
-// Lane of the upper-triangle entry (i, k), i <= k < 6, in the solve's layout.
-__device__ __forceinline__ int upper_lane(int i, int k) { return i * (11 - i) / 2 + k; }
-
-// Eq. 5: (A^T A + 2 lambda n P^T P) x = A^T b, P = [I3 | 0];
-// T <- [Exp(alpha, beta, gamma) | t] T, and the float32 transforms of the new
-// T. FP64, run by one warp, on values alone (S: the 29 sums in shared memory;
-// Tc: lane 4 i + j < 12 holds column j of T; Tmc: a lane o >= 12 holds the
-// column of Tm that its transform entry o needs, Tmt Tm's translation; gadd:
-// what lane 21 + r < 24 adds to its right-hand side).
-//
-// What bounds it is the chain of dependent FP64 operations (~64 cycles each on
-// this part), not their number, so the chain is kept short: lane (r, c) holds
-// one entry of the upper triangle, lane 21 + r the right-hand side, and step j
-// of a Gauss-Jordan elimination is one broadcast of the pivot, one reciprocal
-// and one fused multiply-add for all entries at once (the products H_rj H_jc
-// need no reciprocal and run beside it); eliminating above the pivot too
-// leaves no back substitution. A diagonal lane's last value is its pivot: the
-// system is degenerate when one is not above 1e-12 of its own entry of H.
-// Measured on GB300: 8.5 us for the Cholesky factorisation and substitutions
-// by one thread that this replaces, 3.9 us with this form (a 640x480 pair).
-struct Solved {
-  double x;     // lanes 21..26: the increment (alpha, beta, gamma, tx, ty, tz)
-  double T;     // lanes 0..11: the new pose, row-major
-  float xf;     // lanes 0..23: its float32 transforms (see xf_entry)
-  bool degenerate;
-};
-
-__device__ __forceinline__ Solved solve_lanes(const double* S, double reg, const double (&Tc)[3],
-                                              const double (&Tmc)[3], const double (&Tmt)[3],
-                                              double gadd) {
-  const int lane = threadIdx.x & 31;
-  const bool rhs = lane >= 21;
-  const int r = rhs ? min(lane - 21, 5)
-                    : (lane >= 6) + (lane >= 11) + (lane >= 15) + (lane >= 18) + (lane >= 20);
-  const int c = rhs ? 6 : lane - upper_lane(r, 0);
-  double h = S[min(lane, 26)] + (rhs ? gadd : (r == c && r < 3 ? reg : 0.0));
-  const double h0 = h;
-  double pinv = 0.0;
-#pragma unroll
-  for (int j = 0; j < 6; ++j) {
-    const double piv = lane_of(h, upper_lane(j, j));
-    const double a = lane_of(h, r > j ? upper_lane(j, r) : upper_lane(r, j));
-    const double b = lane_of(h, rhs ? 21 + j : upper_lane(j, max(c, j)));
-    const double ab = a * b;
-    const double ri = recip(piv);
-    if (r == j) pinv = ri;
-    else if (c > j) h = fma(-ab, ri, h);
-  }
-  Solved o;
-  o.degenerate = __any_sync(0xffffffffu, !rhs && r == c && !(h > 1e-12 * h0));
-  o.x = h * pinv;
-  const double w0 = lane_of(o.x, 21), w1 = lane_of(o.x, 22), w2 = lane_of(o.x, 23);
-  // Rodrigues: dR = I + A [w]x + B [w]x^2, A = sin(t)/t, B = (1 - cos t)/t^2;
-  // below t = 0.2 both from their Taylor series (truncation < 3e-15), A in the
-  // even lanes and B in the odd ones
-  const double th2 = fma(w2, w2, fma(w1, w1, w0 * w0));
-  double A, B;
-  if (th2 < 0.04) {
-    const bool odd = lane & 1;
-    double f = fma(th2, odd ? 1.0 / 3628800.0 : 1.0 / 362880.0, odd ? -1.0 / 40320.0 : -1.0 / 5040.0);
-    f = fma(th2, f, odd ? 1.0 / 720.0 : 1.0 / 120.0);
-    f = fma(th2, f, odd ? -1.0 / 24.0 : -1.0 / 6.0);
-    f = fma(th2, f, odd ? 0.5 : 1.0);
-    A = lane_of(f, 0);
-    B = lane_of(f, 1);
-  } else {
-    const double th = sqrt(th2);
-    double sn, cs;
-    sincos(th, &sn, &cs);
-    A = sn / th;
-    B = (1.0 - cs) / th2;
-  }
-  // lane 4 i + k: dR(i, k), with [w]x(i, k) = -+ the third component (+ where
-  // k is two after i) and [w]x^2 = w w^T - t^2 I; then lane 4 i + j: row i of
-  // dR times column j of T
-  const int i = min(lane >> 2, 2), j = lane & 3;
-  const double wi = i == 0 ? w0 : (i == 1 ? w1 : w2);
-  const double wk = j == 0 ? w0 : (j == 1 ? w1 : w2);
-  const int m = 3 - i - j;
-  const double wm = m == 0 ? w0 : (m == 1 ? w1 : w2);
-  const double K = i == j ? 0.0 : ((j - i + 3) % 3 == 2 ? wm : -wm);
-  const double dR = fma(B, fma(wi, wk, i == j ? -th2 : 0.0), fma(A, K, i == j ? 1.0 : 0.0));
-  double t = lane_of(o.x, 24 + i);
-  t = j == 3 ? t : 0.0;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) t = fma(lane_of(dR, 4 * i + k), Tc[k], t);
-  o.T = t;
-  // entry o of the float32 transforms, operation for operation as xf_entry
-  const int q = max(lane - 12, 0);
-  const int ej = q < 9 ? q % 3 : 3;
-  const double rel = j == 3 ? __dsub_rn(t, i == 0 ? Tmt[0] : (i == 1 ? Tmt[1] : Tmt[2])) : t;
-  double s = __dmul_rn(Tmc[0], lane_of(rel, ej));
-  s = __dadd_rn(s, __dmul_rn(Tmc[1], lane_of(rel, 4 + ej)));
-  s = __dadd_rn(s, __dmul_rn(Tmc[2], lane_of(rel, 8 + ej)));
-  const double own = lane_of(t, lane < 9 ? (lane / 3) * 4 + lane % 3 : (lane < 12 ? (lane - 9) * 4 + 3 : 0));
-  o.xf = __double2float_rn(lane < 12 ? own : s);
-  return o;
-}
-
-// The column of Tm that transform entry `lane` needs, and Tm's translation.
-__device__ __forceinline__ void load_tm(const double* Tm, double (&Tmc)[3], double (&Tmt)[3]) {
-  const int q = max((int)(threadIdx.x & 31) - 12, 0);
-  const int ei = q < 9 ? q / 3 : min(q - 9, 2);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    Tmc[k] = Tm[4 * k + ei];
-    Tmt[k] = Tm[4 * k + 3];
-  }
-}
-
-// The prior-anchored variant's addition to the right-hand side, -2 lambda n r,
-// r = log(R R_prior^T), in lanes 21..23 (0 elsewhere): M = R R_prior^T one
-// entry per lane, then t = atan2(|v| / 2, (tr M - 1) / 2) and
-// r = t / (2 sin t) v, v = (M21 - M12, M02 - M20, M10 - M01).
-__device__ double anchored_rhs(const double* T, const double* prior_R, double reg) {
-  const int lane = threadIdx.x & 31;
-  double m = 0.0;
-  if (lane < 9)
-    for (int k = 0; k < 3; ++k) m += __ldcg(T + (lane / 3) * 4 + k) * __ldcg(prior_R + (lane % 3) * 3 + k);
-  const double v0 = lane_of(m, 7) - lane_of(m, 5), v1 = lane_of(m, 2) - lane_of(m, 6),
-               v2 = lane_of(m, 3) - lane_of(m, 1);
-  const double sn = 0.5 * sqrt(v0 * v0 + v1 * v1 + v2 * v2);
-  const double cs = 0.5 * (lane_of(m, 0) + lane_of(m, 4) + lane_of(m, 8) - 1.0);
-  const double t = atan2(sn, cs);
-  const double f = t < 1e-4 ? 0.5 * (1.0 + t * t / 6.0) : t / (2.0 * sn);
-  return lane == 21 ? -reg * f * v0 : lane == 22 ? -reg * f * v1 : lane == 23 ? -reg * f * v2 : 0.0;
-}
-
-// The solve and update of one pair (solve_lanes) and its bookkeeping:
-// convergence control (Sec. 3.4), the next iteration's window, the trace.
-// Run by one warp; pre: the pair's state from load_pre, valid in lane 0.
-// Returns (in lane 0) the level the pair iterates at next, or -1 when it has
-// finished or stopped.
+// solve_update for the launches whose pair state lies in memory that other
+// blocks wrote.
 __device__ __noinline__ int solve_update_warp(const PairDesc* d, PairState* st, const double* S,
                                                int level, const KParams& P, int passes,
                                                const PairPre& pre) {
-  const int lane = threadIdx.x & 31;
-  const unsigned long long t_start = globaltimer_ns();
-  const int n = (int)S[27];
-  if (n < P.n_min) {
-    if (lane == 0) {
-      st->status = KF_ERR_TOO_FEW_INLIERS;
-      st->stopped = 1;
-    }
-    return -1;
-  }
-  double Tc[3], Tmc[3], Tmt[3];
+  double Tc[3];
 #pragma unroll
-  for (int k = 0; k < 3; ++k) Tc[k] = __ldcg(&st->T[4 * k + (lane & 3)]);
-  load_tm(d->Tm, Tmc, Tmt);
-  const double lam = lane_of(lane == 0 ? lambda_of_n(P.lambda_mode, pre.lambda_c, n) : 0.0, 0);
-  const double reg = (2.0 * lam) * (double)n;
-  double gadd = 0.0;
-  if ((P.flags & KF_PRIOR_ANCHORED) && __shfl_sync(0xffffffffu, pre.has_prior, 0))
-    gadd = anchored_rhs(st->T, st->prior_R, reg);
-  const Solved o = solve_lanes(S, reg, Tc, Tmc, Tmt, gadd);
-  if (o.degenerate) {
-    if (lane == 0) {
-      st->status = KF_ERR_DEGENERATE;
-      st->stopped = 1;
-    }
-    return -1;
-  }
-  if (lane < 12) st->T[lane] = o.T;
-  if (lane < 24) st->xf[lane] = o.xf;
-  double x[6];
-#pragma unroll
-  for (int i = 0; i < 6; ++i) x[i] = lane_of(o.x, 21 + i);
-  if (lane != 0) return -1;
-  // bookkeeping (the state's fields from pre)
-  const int kmed = pre.kmed, N = pre.N, it = pre.it, tl = pre.tl;
-  if (tl < KF_TRACE_MAX) {
-    kf_iter_record& r = st->trace[tl];
-    st->trace_len = tl + 1;
-    r.level = level;
-    r.iter = it;
-    r.N = N;
-    r.kmed = kmed;
-    r.klo = pre.klo;
-    r.khi = pre.khi;
-    r.n = n;
-    r.passes = passes;
-    r.w0 = pre.w0;
-    r.w1 = pre.w1;
-    r.pad = 0;
-    r.lambda = lam;
-    for (int i = 0; i < 6; ++i) r.x[i] = x[i];
-    r.solve_ns = (int)(globaltimer_ns() - t_start);
-  }
-  st->iters[level] = it + 1;
-  st->total_iters = pre.total + 1;
-  st->median_bin[level] = kmed;
-  st->valid_pairs = N;
-  st->inliers = n;
-  st->sb2 = S[28];
-  int hl = pre.hl;
-  int kh[kMaxWindow];
-  for (int i = 0; i < kMaxWindow; ++i) kh[i] = pre.kh[i];
-  if (hl < kMaxWindow) {
-    kh[hl++] = kmed;
-  } else {
-    for (int i = 0; i + 1 < kMaxWindow; ++i) kh[i] = kh[i + 1];
-    kh[kMaxWindow - 1] = kmed;
-  }
-  bool conv = false;
-  if ((P.flags & KF_USE_CONVERGENCE) && hl >= P.conv_window) {
-    conv = true;
-    for (int i = hl - P.conv_window; i < hl; ++i) conv = conv && kh[i] == kmed;
-  }
-  int cur = level;
-  if (conv || it + 1 >= P.caps[level]) {
-    if (level == 0 && (P.flags & KF_USE_CONVERGENCE) && !conv && pre.status == KF_OK)
-      st->status = KF_NOT_CONVERGED;
-    cur = level - 1;
-    hl = 0;
-  }
-  st->cur_level = cur;
-  st->hist_len = hl;
-  for (int i = 0; i < kMaxWindow; ++i) st->kmed_hist[i] = kh[i];
-  // the next iteration's band-edge window around this band edge
-  int w0 = -1, w1 = -1;
-  if (P.split_ok && cur >= 0) {
-    const int below = cur == level ? P.win_same_below : P.win_next_below;
-    const int above = cur == level ? P.win_same_above : P.win_next_above;
-    w0 = max(0, pre.khi - below + 1);
-    w1 = pre.khi + above + 1;
-  }
-  st->w0 = w0;
-  st->w1 = w1;
-  return cur;
+  for (int k = 0; k < 3; ++k) Tc[k] = __ldcg(&st->T[4 * k + (threadIdx.x & 3)]);
+  return solve_update(d, st, S, level, P, passes, pre, Tc, [](const Solved&, int, int, int) {});
 }
 
 // ---------------------------------------------------------------------------
 // Active work list (see kf_internal.cuh for the layout).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ int items_of(const PairDesc* d, int level) {
-  const int px = d->lv[level].fw * d->lv[level].fh;
-  const int c = level_chunk(level);
-  return (px + c - 1) / c;
-}
-
 // Block-wide exclusive scan of one int per thread (kBlock threads); returns the
 // exclusive prefix and writes the block total to *total.
 __device__ int block_exclusive_scan(int v, int* total) {
@@ -669,302 +196,12 @@ __device__ __forceinline__ int find_slot(const int* prefix, int npairs, int f) {
   return lo;
 }
 
-// Row of Eq. 3 for the pair (p, q, n): a = [(p x n)^T, n^T], b = n . (q - p),
-// accumulated into the 29 sums (21 upper a a^T, 6 a b, n, b^2). Every
-// operation is written out (products and fused multiply-adds explicitly), so
-// that each kernel that inlines it rounds the same way.
-__device__ __forceinline__ void ls_row(const float* p, const float* q, const float* n, float* a,
-                                       float& b) {
-  a[0] = fmaf(p[1], n[2], -__fmul_rn(p[2], n[1]));
-  a[1] = fmaf(p[2], n[0], -__fmul_rn(p[0], n[2]));
-  a[2] = fmaf(p[0], n[1], -__fmul_rn(p[1], n[0]));
-  a[3] = n[0];
-  a[4] = n[1];
-  a[5] = n[2];
-  b = fmaf(n[0], __fsub_rn(q[0], p[0]),
-           fmaf(n[1], __fsub_rn(q[1], p[1]), __fmul_rn(n[2], __fsub_rn(q[2], p[2]))));
-}
-
-// Registers of a thread's running sums: the 29 sums, and with KF_KAHAN their
-// 29 compensations after them.
-constexpr int kSumRegs = KF_KAHAN ? 2 * kSums : kSums;
-
-// Sum k += x y. Plain: one fused multiply-add. KF_KAHAN: compensated
-// summation (Kahan, 1965); sum[kSums + k] holds c, the rounding error of the
-// last addition, which the next term has subtracted before it is added
-// (x y - c in one fused rounding); the sum's value is then sum[k] - c.
-__device__ __forceinline__ void add_term(float* sum, int k, float x, float y) {
-#if KF_KAHAN
-  const float t = fmaf(x, y, -sum[kSums + k]);
-  const float s = __fadd_rn(sum[k], t);
-  sum[kSums + k] = __fsub_rn(__fsub_rn(s, sum[k]), t);
-  sum[k] = s;
-#else
-  sum[k] = fmaf(x, y, sum[k]);
-#endif
-}
-
-__device__ __forceinline__ void accumulate(const float* a, float b, float* sum) {
-  int s = 0;
-#pragma unroll
-  for (int r = 0; r < 6; ++r)
-#pragma unroll
-    for (int c = r; c < 6; ++c) {
-      add_term(sum, s, a[r], a[c]);
-      ++s;
-    }
-#pragma unroll
-  for (int r = 0; r < 6; ++r) add_term(sum, 21 + r, a[r], b);
-  sum[27] = __fadd_rn(sum[27], 1.f);  // a count: exact below 2^24
-  add_term(sum, 28, b, b);
-}
-
-constexpr int kPassHist = 0, kPassSplit = 1, kPassBand = 2;
-
-// ---------------------------------------------------------------------------
-// Association passes. A batch is kBatch = KF_ASSOC_U * kBlock consecutive
-// frame pixels of one item; thread t takes pixels b0 + t + u kBlock
-// (u < KF_ASSOC_U): its frame vertices (coalesced loads), their projections,
-// then every model gather of the batch issued before any is used. Warps run
-// their batches independently (no barrier inside an item). Measured on GB300
-// at 640x480: four pixels per thread and no software pipeline across
-// batches beat one or two pixels per thread with the next batch's gathers in
-// flight (the pipeline's second batch of registers costs the pixels in flight
-// that hide the gathers), and beat staging the frame vertices in shared
-// memory with bulk copies (a block barrier per batch).
-// ---------------------------------------------------------------------------
-constexpr int kU = KF_ASSOC_U;
-constexpr int kBatch = kU * kBlock;
-
-// The 24 float32 transform entries, read from shared memory once per batch
-// (volatile: the loads stay inside the batch, so the registers holding them
-// are free again while the gathers are awaited and the sums accumulate).
-// sxf must be a shared-memory array aligned to 16 bytes (vector loads).
-__device__ __forceinline__ void load_xf(const float* sxf, float* x) {
-  const unsigned a = (unsigned)__cvta_generic_to_shared(sxf);
-#pragma unroll
-  for (int c = 0; c < 6; ++c)
-    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                 : "=f"(x[4 * c]), "=f"(x[4 * c + 1]), "=f"(x[4 * c + 2]), "=f"(x[4 * c + 3])
-                 : "r"(a + 16 * c));
-}
-
-struct Verts {  // one batch's frame vertices (NaN past the batch's end)
-  float v[kU][3];
-};
-
-template <bool kGate>
-struct Batch {  // one batch after association, its gathers in flight
-  float p[kU][3], q[kU][3], nq[kU][3];
-  float nf[kGate ? kU : 1][3];  // frame normals (angle gate)
-  int j[kU];
-};
-
-__device__ __forceinline__ void prefetch_l2(const void* p) {
-  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
-}
-__device__ __forceinline__ void prefetch_l1(const void* p) {
-  asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
-}
-__device__ __forceinline__ void prefetch_line(const void* p) {
-  if constexpr (KF_PREFETCH >= 3) prefetch_l1(p);
-  else prefetch_l2(p);
-}
-
-// Hints for the warp's next batch [nb0, ne): its frame-vertex lines (lanes
-// 0..3 u: one line of 32 pixels per plane each) and, with an offset `off`
-// (model index minus frame index of a pixel this warp just matched), the
-// model vertex and normal lines at that offset. Every address stays inside
-// its plane.
-template <class T>
-__device__ __forceinline__ void prefetch_next(const LevelMaps& L, int nb0, int ne, int off) {
-  if constexpr (KF_PREFETCH == 0) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int kLines = 3 * kU * (KF_PREFETCH == 2 || KF_PREFETCH == 4 ? 3 : 1);
-  for (int q = lane; q < kLines; q += 32) {
-    const int set = q / (3 * kU);  // 0: frame vertex, 1: model vertex, 2: model normal
-    const int r = q - set * 3 * kU, c = r / kU, u = r - c * kU;
-    const int i = nb0 + warp * 32 + u * kBlock;
-    if (i >= ne) continue;
-    if (set == 0) {
-      prefetch_line(static_cast<const T*>(L.fV) + (size_t)c * L.fps + i);
-    } else {
-      const int mn = L.mw * L.mh;
-      const int j = min(max(i + off, 0), mn - 1);
-      prefetch_line(static_cast<const T*>(set == 1 ? L.mV : L.mN) + (size_t)c * mn + j);
-    }
-  }
-}
-
-template <class T>
-__device__ __forceinline__ void load_verts(const LevelMaps& L, int b0, int e, Verts& V) {
-  const T* fV = static_cast<const T*>(L.fV);
-  const int fs = L.fps;
-#pragma unroll
-  for (int u = 0; u < kU; ++u) {
-    const int i = b0 + threadIdx.x + u * kBlock;
-    const bool in = i < e;
-    const int ii = in ? i : 0;
-    const float x = Store<T>::ld(fV, ii), y = Store<T>::ld(fV, fs + ii), z = Store<T>::ld(fV, 2 * fs + ii);
-    V.v[u][0] = in ? x : __int_as_float(0x7fc00000);
-    V.v[u][1] = y;
-    V.v[u][2] = z;
-  }
-}
-
-// Projective association (Sec. 3.2; normal shooting with kAShoot) of a batch:
-// world points, matched model pixels, and the gathers of their model vertex
-// (and normal, when the pass or the gate needs it) issued.
-template <class T, int kA, int kPass>
-__device__ __forceinline__ void associate_batch(const LevelMaps& L, int b0, const Verts& V,
-                                                const float* sxf, const KParams& P,
-                                                Batch<(kA & kAGate) != 0>& B) {
-  constexpr bool kGate = (kA & kAGate) != 0;
-  constexpr bool kNeedN = kGate || kPass != kPassHist;
-  const int fs = L.fps, mn = L.mw * L.mh;
-  const T* mV = static_cast<const T*>(L.mV);
-  const T* mN = static_cast<const T*>(L.mN);
-  float xf[24];
-  load_xf(sxf, xf);
-#pragma unroll
-  for (int u = 0; u < kU; ++u) B.j[u] = project(L, V.v[u][0], V.v[u][1], V.v[u][2], xf, B.p[u]);
-  if constexpr (kGate || (kA & kAShoot) != 0) {
-    const T* fN = static_cast<const T*>(L.fN);
-#pragma unroll
-    for (int u = 0; u < kU; ++u) {
-      const int i = B.j[u] >= 0 ? b0 + threadIdx.x + u * kBlock : 0;
-      const float nf[3] = {Store<T>::ld(fN, i), Store<T>::ld(fN, fs + i), Store<T>::ld(fN, 2 * fs + i)};
-      if constexpr (kGate) {
-        B.nf[u][0] = nf[0];
-        B.nf[u][1] = nf[1];
-        B.nf[u][2] = nf[2];
-      }
-      if constexpr ((kA & kAShoot) != 0) {
-        if (B.j[u] >= 0) {
-          const float nw[3] = {rot3(xf + 0, nf[0], nf[1], nf[2]), rot3(xf + 3, nf[0], nf[1], nf[2]),
-                               rot3(xf + 6, nf[0], nf[1], nf[2])};
-          B.j[u] = shoot(L, mV, B.j[u], B.p[u], nw, P.shoot_w, B.q[u]);
-        }
-      }
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < kU; ++u) {
-    const int jj = B.j[u] < 0 ? 0 : B.j[u];
-    if constexpr ((kA & kAShoot) == 0) {
-      B.q[u][0] = Store<T>::ld(mV, jj);
-      B.q[u][1] = Store<T>::ld(mV, mn + jj);
-      B.q[u][2] = Store<T>::ld(mV, 2 * mn + jj);
-    }
-    if constexpr (kNeedN) {
-      B.nq[u][0] = Store<T>::ld(mN, jj);
-      B.nq[u][1] = Store<T>::ld(mN, mn + jj);
-      B.nq[u][2] = Store<T>::ld(mN, 2 * mn + jj);
-    }
-  }
-}
-
-// What an association pass does with a batch once its gathers have landed:
-// the point-to-point distance, bin and gates, then
-//  kPassHist   the distance histogram only (no band-edge window is known);
-//  kPassSplit  the histogram, and the rows of the pixels with bin < lo (= w0)
-//              summed in registers, the rows of the pixels with bin in
-//              [lo, hi) (= [w0, w1)) written as 32-byte records, packed in
-//              the warp's record region of the item (rbase; wc counts the
-//              records the warp has written there, in pixel order);
-//  kPassBand   no histogram: the rows of the pixels with bin in [lo, hi]
-//              (= the band [klo, khi]) summed in registers.
-// kMode 1 also writes the inspection outputs (model pixel and bin per pixel).
-template <int kA, int kPass, int kMode>
-__device__ __forceinline__ void finish_batch(const PairDesc* d, int b0, int e,
-                                             const Batch<(kA & kAGate) != 0>& B, const float* sxf,
-                                             const KParams& P, unsigned* sh_hist, int lo, int hi,
-                                             float* sum, int rbase, int& wc) {
-  constexpr bool kGate = (kA & kAGate) != 0;
+// Writes the warp's row of item li's partial, in slot A or slot B.
+__device__ __forceinline__ void write_row(const PairDesc* d, int li, bool slot_b, const float* sum) {
+  const float v = warp_sums(sum);
   const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int u = 0; u < kU; ++u) {
-    const int i = b0 + threadIdx.x + u * kBlock;
-    int k = B.j[u] >= 0 ? bin_of(B.p[u], B.q[u], P) : -1;
-    if constexpr (kGate) {
-      if (k >= 0 && !angle_ok(sxf, B.nf[u], B.nq[u], P)) k = -1;
-    }
-    if constexpr (kPass != kPassBand) {
-      if constexpr (kMode == 1) {
-        if (i < e) {
-          d->dbg_index[i] = k >= 0 ? B.j[u] : -1;
-          d->dbg_bin[i] = k;
-        }
-      }
-      if (k >= 0) atomicAdd(sh_hist + k, 1u);
-    }
-    if constexpr (kPass == kPassSplit) {
-      bool win = false;
-      float a[6], b;
-      if (k >= 0 && k < hi) {
-        ls_row(B.p[u], B.q[u], B.nq[u], a, b);
-        if (k < lo) accumulate(a, b, sum);
-        else win = true;
-      }
-      // the window pixels of these 32 lanes take the next places of the
-      // warp's region, in lane order
-      const unsigned m = __ballot_sync(0xffffffffu, win);
-      if (win) {
-        const int r = rbase + wc + __popc(m & ((1u << lane) - 1u));
-        KF_GUARD(r < d->px_cap + kChunk, 6, r, d->px_cap)
-        {
-          float4* rec = d->recs + 2 * (size_t)r;
-          rec[0] = make_float4(a[0], a[1], a[2], a[3]);
-          rec[1] = make_float4(a[4], a[5], b, __int_as_float(k));
-        }
-      }
-      wc += __popc(m);
-    }
-    if constexpr (kPass == kPassBand) {
-      if (k >= lo && k <= hi) {
-        float a[6], b;
-        ls_row(B.p[u], B.q[u], B.nq[u], a, b);
-        accumulate(a, b, sum);
-      }
-    }
-  }
-}
-
-// The warp's sum of the 29 per-lane float32 sums of one item, written as the
-// warp's row of the item's partial: recursive halving, at each of five steps
-// a lane keeps half of its remaining values and adds the partner lane's copy
-// of that half (31 shuffles), leaving lane s with the warp's sum s (with
-// KF_KAHAN a lane enters its compensated value, the sum minus its
-// compensation). No block barrier: the warps of a block run their items
-// independently.
-__device__ __forceinline__ void warp_partial(const float* sum, float* dst) {
-  const int lane = threadIdx.x & 31;
-  float v[32];
-#pragma unroll
-  for (int k = 0; k < kSums; ++k) v[k] = KF_KAHAN ? __fsub_rn(sum[k], sum[kSumRegs - kSums + k]) : sum[k];
-#pragma unroll
-  for (int k = kSums; k < 32; ++k) v[k] = 0.f;
-#pragma unroll
-  for (int h = 16; h >= 1; h >>= 1) {
-    const bool upper = (lane & h) != 0;
-#pragma unroll
-    for (int k = 0; k < h; ++k) {
-      const float send = upper ? v[k] : v[k + h];
-      const float keep = upper ? v[k + h] : v[k];
-      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, h);
-    }
-  }
-  if (lane < kSums) dst[(threadIdx.x >> 5) * 32 + lane] = v[0];
-}
-
-// Where item li's partial rows go: slot A or slot B.
-__device__ __forceinline__ float* partial_rows(const PairDesc* d, int li, bool slot_b) {
-  return d->partials + (size_t)li * kPartialStride + (slot_b ? kSlotB : 0);
-}
-
-__device__ __forceinline__ void zero_sums(float* sum) {
-#pragma unroll
-  for (int k = 0; k < kSumRegs; ++k) sum[k] = 0.f;
+  if (lane < kSums)
+    d->partials[(size_t)li * kPartialStride + (slot_b ? kSlotB : 0) + (threadIdx.x >> 5) * 32 + lane] = v;
 }
 
 // An association pass over the items [first, first + run) of one pair, in
@@ -977,8 +214,8 @@ __device__ void assoc_items(const PairDesc* d, const LevelMaps& L, int first, in
   constexpr bool kGate = (kA & kAGate) != 0;
   const int fn = L.fw * L.fh;
   float sum[kSumRegs];
-  Verts va;
-  Batch<kGate> sa;
+  Verts<kU> va;
+  Batch<kGate, kU> sa;
   const int warp = threadIdx.x >> 5;
   for (int li = first; li < first + run; ++li) {
     const int ib = li * chunk, ie = min(fn, ib + chunk);
@@ -991,8 +228,8 @@ __device__ void assoc_items(const PairDesc* d, const LevelMaps& L, int first, in
     // divide the item)
     for (int b0 = ib; b0 < ie; b0 += kBatch) {
       const int e = min(ie, b0 + kBatch);
-      load_verts<T>(L, b0, e, va);
-      associate_batch<T, kA, kPass>(L, b0, va, sxf, P, sa);
+      load_verts<T>(L, b0, e, threadIdx.x, va);
+      associate_batch<T, kA, kPass>(L, b0, threadIdx.x, va, sxf, P, sa);
       {  // L2 hints for this warp's next batch (of this item or the next)
         int nb0 = b0 + kBatch, ne = e + kBatch;
         if (nb0 >= ie) {
@@ -1006,7 +243,7 @@ __device__ void assoc_items(const PairDesc* d, const LevelMaps& L, int first, in
         const int off = __shfl_sync(0xffffffffu, sa.j[0] - (b0 + threadIdx.x), src);
         prefetch_next<T>(L, nb0, ne, ok ? off : 0);
       }
-      finish_batch<kA, kPass, kMode>(d, b0, e, sa, sxf, P, sh_hist, lo, hi, sum, rbase, wc);
+      finish_batch<kA, kPass, kMode>(d, b0, e, threadIdx.x, sa, sxf, P, sh_hist, lo, hi, sum, rbase, wc);
     }
     if constexpr (kPass == kPassSplit) {
       if ((threadIdx.x & 31) == 0) {
@@ -1016,76 +253,22 @@ __device__ void assoc_items(const PairDesc* d, const LevelMaps& L, int first, in
     }
     if constexpr (kPass != kPassHist) {
       KF_GUARD(li < d->partial_cap, 1, li, d->partial_cap)
-      warp_partial(sum, partial_rows(d, li, kPass == kPassBand));
+      write_row(d, li, kPass == kPassBand, sum);
     }
   }
   __syncthreads();
 }
 
-// Reduction pass of an item whose band edge fell in the window: the
-// recorded pixels with klo <= bin <= khi, in registers. Warp w reads the
-// region warp w of the association pass filled: its record count and the
-// first 32 kFixR records in one round trip (places past the count are read
-// and ignored: the region has room for every pixel of the warp, and the
-// buffer a chunk of padding), lane l taking places l, l + 32, ... in order.
-// The records were written by other blocks: read through L2. fix_issue puts
-// an item's loads in flight; fix_consume adds them (and any further rounds).
-constexpr int kFixR = 2;
-struct FixLoad {
-  int total;
-  float4 r0[kFixR], r1[kFixR];
-};
-
-__device__ __forceinline__ void fix_issue(const PairDesc* d, int li, int chunk, FixLoad& f) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int rbase = li * chunk + warp * (chunk / kBlockWarps);
-  [[maybe_unused]] const int cap = chunk / kBlockWarps;  // places of the region
-  KF_GUARD(li < d->partial_cap && rbase + cap <= d->px_cap + kChunk, 11, li, rbase) {}
-  f.total = lane == 0 && li < d->partial_cap ? (int)__ldcg(d->wcount + li * kBlockWarps + warp) : 0;
-#pragma unroll
-  for (int r = 0; r < kFixR; ++r) {
-    const size_t i = (size_t)rbase + r * 32 + lane;
-    f.r0[r] = __ldcg(d->recs + 2 * i);
-    f.r1[r] = __ldcg(d->recs + 2 * i + 1);
-  }
-}
-
-__device__ __forceinline__ void fix_consume(const PairDesc* d, int li, int chunk, int klo, int khi,
-                                            FixLoad& f, float* sum) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int rbase = li * chunk + warp * (chunk / kBlockWarps);
-  [[maybe_unused]] const int cap = chunk / kBlockWarps;
-  int total = __shfl_sync(0xffffffffu, f.total, 0);
-  KF_GUARD(total <= cap, 10, total, cap) {}
-#ifdef KF_CHECKED
-  total = min(total, cap);
-#endif
-  for (int e0 = 0;;) {
-#pragma unroll
-    for (int r = 0; r < kFixR; ++r) {
-      if (e0 + r * 32 + lane >= total) continue;
-      const int k = __float_as_int(f.r1[r].w);
-      if (k >= klo && k <= khi) {
-        const float a[6] = {f.r0[r].x, f.r0[r].y, f.r0[r].z, f.r0[r].w, f.r1[r].x, f.r1[r].y};
-        accumulate(a, f.r1[r].z, sum);
-      }
-    }
-    e0 += 32 * kFixR;
-    if (e0 >= total) break;
-#pragma unroll
-    for (int r = 0; r < kFixR; ++r) {
-      const size_t i = (size_t)rbase + e0 + r * 32 + lane;
-      f.r0[r] = __ldcg(d->recs + 2 * i);
-      f.r1[r] = __ldcg(d->recs + 2 * i + 1);
-    }
-  }
+__device__ __forceinline__ int record_count(const PairDesc* d, int li) {
+  return li < d->partial_cap ? (int)__ldcg(d->wcount + li * kBlockWarps + (threadIdx.x >> 5)) : 0;
 }
 
 __device__ __forceinline__ void fixup_item(const PairDesc* d, int li, int chunk, int klo, int khi,
                                            float* sum) {
   FixLoad f;
-  fix_issue(d, li, chunk, f);
-  fix_consume(d, li, chunk, klo, khi, f, sum);
+  f.total = record_count(d, li);
+  fix_issue(d, li, chunk, threadIdx.x >> 5, f);
+  fix_consume(d, li, chunk, threadIdx.x >> 5, klo, khi, f, sum);
 }
 
 // The reduction pass of a hit over every item of a pair by one block (the
@@ -1095,15 +278,22 @@ __device__ __forceinline__ void fixup_item(const PairDesc* d, int li, int chunk,
 // would write (the same warp-to-region map, the same order): which way runs
 // changes no bit. Block-wide: ends with a barrier.
 __device__ __noinline__ void fixup_all(const PairDesc* d, int count, int chunk, int klo, int khi) {
+  const int warp = threadIdx.x >> 5;
   FixLoad cur, nxt = {};
-  if (count > 0) fix_issue(d, 0, chunk, cur);
+  if (count > 0) {
+    cur.total = record_count(d, 0);
+    fix_issue(d, 0, chunk, warp, cur);
+  }
   for (int li = 0; li < count; ++li) {
-    if (li + 1 < count) fix_issue(d, li + 1, chunk, nxt);
+    if (li + 1 < count) {
+      nxt.total = record_count(d, li + 1);
+      fix_issue(d, li + 1, chunk, warp, nxt);
+    }
     float sum[kSumRegs];
     zero_sums(sum);
-    fix_consume(d, li, chunk, klo, khi, cur, sum);
+    fix_consume(d, li, chunk, warp, klo, khi, cur, sum);
     KF_GUARD(li < d->partial_cap, 1, li, d->partial_cap)
-    warp_partial(sum, partial_rows(d, li, true));
+    write_row(d, li, true, sum);
     cur = nxt;
   }
   __threadfence_block();
@@ -1123,7 +313,7 @@ __device__ void reduce_items(const PairDesc* d, const LevelMaps& L, int first, i
       zero_sums(sum);
       fixup_item(d, li, chunk, klo, khi, sum);
       KF_GUARD(li < d->partial_cap, 1, li, d->partial_cap)
-      warp_partial(sum, partial_rows(d, li, true));
+      write_row(d, li, true, sum);
     } else {
       assoc_items<T, kA, kPassBand, 0>(d, L, li, 1, chunk, sxf, P, nullptr, klo, khi);
     }
@@ -1131,14 +321,13 @@ __device__ void reduce_items(const PairDesc* d, const LevelMaps& L, int first, i
 }
 
 // The pair's reduction epilogue (block-wide, run by the block that finished
-// its last item): per sum, the items' partials in FP64 in a fixed order (slot
-// A + slot B on a hit, slot B alone otherwise; 8 strided sub-sums, then a tree
-// over the 8), the histogram cleared for the next iteration, then the solve and
+// its last item): per sum, the items' partials in a fixed order (slot A +
+// slot B on a hit, slot B alone otherwise; 8 strided sub-sums, then the 8), the histogram cleared for the next iteration, then the solve and
 // update (mode 2: the sums are stored instead). Returns (in thread 0) the
 // solve's next level (-1: finished or stopped).
 __device__ __noinline__ int combine_and_solve(const PairDesc* d, PairState* st, int count,
                                                int level, const KParams& P, int mode,
-                                               double (*s_part)[kSums], double* s_sums) {
+                                               ItemSum (*s_part)[kSums], double* s_sums) {
   __shared__ int s_hit;
   PairPre pre;
   if (threadIdx.x == 0) {
@@ -1153,10 +342,8 @@ __device__ __noinline__ int combine_and_solve(const PairDesc* d, PairState* st, 
   const int hit = s_hit;
   // warp `sub` takes items sub, sub + 8, ...; lane k < 29 sums, per item, the
   // 16 rows of sum k (slot A's 8 warps, zero on a miss, and slot B's) in
-  // float32 by pairwise halving, then adds the items in float64, four at a
-  // time (their loads in flight together) as a tree, in increasing order. (The FP64 pipe of this part retires
-  // about two additions per cycle per SM: a float64 chain over every row
-  // would hold the pair's epilogue for microseconds.)
+  // float32 by pairwise halving, then adds the items in increasing order
+  // (ItemSum), four items' loads in flight
   const int k = threadIdx.x & 31, sub = threadIdx.x >> 5;
   auto item_value = [&](int l) {
     const float* a = d->partials + (size_t)l * kPartialStride + k;
@@ -1172,28 +359,25 @@ __device__ __noinline__ int combine_and_solve(const PairDesc* d, PairState* st, 
       for (int i = 0; i < h; ++i) v[i] = __fadd_rn(v[i], v[i + h]);
     return v[0];
   };
-  double t = 0.0;
+  const int shift = sum_shift(count);
+  ItemSum t;
   if (k < kSums) {
     int l = sub;
     for (; l + 24 < count; l += 32) {
       const float e0 = item_value(l), e1 = item_value(l + 8), e2 = item_value(l + 16),
                   e3 = item_value(l + 24);
-      t += ((double)e0 + (double)e1) + ((double)e2 + (double)e3);
+      t.add(e0, shift);
+      t.add(e1, shift);
+      t.add(e2, shift);
+      t.add(e3, shift);
     }
-    for (; l < count; l += 8) t += (double)item_value(l);
+    for (; l < count; l += 8) t.add(item_value(l), shift);
+    s_part[sub][k] = t;
   }
-  if (k < kSums) s_part[sub][k] = t;
   for (int b = threadIdx.x; b < P.bins; b += kBlock) d->hist[b] = 0u;
   __syncthreads();
   if (threadIdx.x < kSums) {
-    double v[kBlockWarps];
-#pragma unroll
-    for (int i = 0; i < kBlockWarps; ++i) v[i] = s_part[i][threadIdx.x];
-#pragma unroll
-    for (int h = 1; h < kBlockWarps; h <<= 1)
-#pragma unroll
-      for (int i = 0; i < kBlockWarps; i += 2 * h) v[i] += v[i + h];
-    s_sums[threadIdx.x] = v[0];
+    s_sums[threadIdx.x] = total_of(s_part, threadIdx.x, shift);
   }
   __syncthreads();
   int next = -1;
@@ -1293,7 +477,8 @@ __global__ void __launch_bounds__(kBlock, KF_REDUCE_MINB) k_reduce_solve(const P
   __shared__ __align__(16) float sxf[24];  // 16-byte vector loads (load_xf)
   __shared__ int s_active, s_klo, s_khi, s_hit, s_last;
   __shared__ double s_sums[kSums];
-  __shared__ double s_part[8][kSums];
+  __shared__ ItemSumWord s_part_raw[8][kSums];
+  ItemSum (*s_part)[kSums] = reinterpret_cast<ItemSum (*)[kSums]>(s_part_raw);
   const int n_items = __ldcg(list);
   const int M = (n_items + gridDim.x - 1) / gridDim.x;
   int f = blockIdx.x * M;
@@ -1354,39 +539,6 @@ __global__ void __launch_bounds__(kBlock, KF_REDUCE_MINB) k_reduce_solve(const P
 // Seed (one block for all pairs, then the first active list), finish, and
 // inspection set-up.
 // ---------------------------------------------------------------------------
-// Initial state of one pair (thread-level; T: the seed pose, 12 doubles).
-__device__ void init_state(const PairDesc* d, const PairInput& pi, const KParams& P, double* sT) {
-  PairState* st = d->st;
-  // T0 = [R_prior | t_init] when the IMU prior is used (Sec. 3), else init
-  for (int i = 0; i < 3; ++i)
-    for (int j = 0; j < 4; ++j) sT[i * 4 + j] = pi.init[i * 4 + j];
-  if (pi.has_prior && (P.flags & KF_USE_PRIOR))
-    for (int i = 0; i < 3; ++i)
-      for (int j = 0; j < 3; ++j) sT[i * 4 + j] = pi.prior_R[i * 3 + j];
-  for (int i = 0; i < 12; ++i) st->T[i] = sT[i];
-  for (int i = 0; i < 9; ++i) st->prior_R[i] = pi.prior_R[i];
-  st->has_prior = pi.has_prior;
-  st->lambda_c = pi.lambda;
-  st->cur_level = P.levels - 1;
-  st->stopped = 0;
-  st->status = KF_OK;
-  for (int l = 0; l < KF_MAX_LEVELS; ++l) {
-    st->iters[l] = 0;
-    st->median_bin[l] = -1;
-  }
-  for (int i = 0; i < kMaxWindow; ++i) st->kmed_hist[i] = 0;
-  st->total_iters = 0;
-  st->hist_len = 0;
-  st->N = st->kmed = st->klo = st->khi = 0;
-  st->w0 = st->w1 = -1;  // no band edge known yet: the first pass is histogram only
-  st->hit = 0;
-  st->valid_pairs = st->inliers = 0;
-  st->sb2 = 0.0;
-  st->trace_len = 0;
-  d->counters[0] = 0u;
-  d->counters[1] = 0u;
-}
-
 __global__ void __launch_bounds__(kBlock) k_icp_init(const PairDesc* const* descs,
                                                      const PairInput* in, int n, int* list,
                                                      KParams P) {
@@ -1405,21 +557,7 @@ __global__ void __launch_bounds__(kBlock) k_icp_init(const PairDesc* const* desc
 }
 
 __global__ void k_icp_finish(const PairDesc* const* descs, PairOutput* out) {
-  const PairDesc* d = descs[blockIdx.x];
-  const PairState* st = d->st;
-  PairOutput& o = out[blockIdx.x];
-  for (int i = 0; i < 12; ++i) o.pose[i] = st->T[i];
-  o.pose[12] = o.pose[13] = o.pose[14] = 0.0;
-  o.pose[15] = 1.0;
-  o.res.status = st->status;
-  for (int l = 0; l < KF_MAX_LEVELS; ++l) {
-    o.res.iters[l] = st->iters[l];
-    o.res.median_bin[l] = st->median_bin[l];
-  }
-  o.res.total_iters = st->total_iters;
-  o.res.inliers = st->inliers;
-  o.res.valid_pairs = st->valid_pairs;
-  o.res.rms_residual = rms_residual(st->sb2, st->inliers);
+  write_output(descs[blockIdx.x], out + blockIdx.x);
 }
 
 __global__ void __launch_bounds__(kBlock) k_debug_setup(const PairDesc* const* self,
@@ -1591,21 +729,7 @@ __device__ void seed_pair(const PairDesc* d, const PairInput& pi, const KParams&
 __device__ void finish_pair(const PairDesc* d, PairOutput* o, int n, unsigned* qh,
                             unsigned long long* qs, unsigned qmask) {
   __shared__ int s_lastpair;
-  if (threadIdx.x == 0) {
-    const PairState* st = d->st;
-    for (int i = 0; i < 12; ++i) o->pose[i] = __ldcg(&st->T[i]);
-    o->pose[12] = o->pose[13] = o->pose[14] = 0.0;
-    o->pose[15] = 1.0;
-    o->res.status = __ldcg(&st->status);
-    for (int l = 0; l < KF_MAX_LEVELS; ++l) {
-      o->res.iters[l] = __ldcg(&st->iters[l]);
-      o->res.median_bin[l] = __ldcg(&st->median_bin[l]);
-    }
-    o->res.total_iters = __ldcg(&st->total_iters);
-    o->res.inliers = __ldcg(&st->inliers);
-    o->res.valid_pairs = __ldcg(&st->valid_pairs);
-    o->res.rms_residual = rms_residual(__ldcg(&st->sb2), __ldcg(&st->inliers));
-  }
+  if (threadIdx.x == 0) write_output(d, o);
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) s_lastpair = atomicAdd(qh + kQDone, 1u) == (unsigned)(n - 1);
@@ -1627,7 +751,8 @@ __global__ void __launch_bounds__(kBlock, KF_SCHED_MINB) k_icp_sched(const PairD
   __shared__ unsigned long long s_word;
   __shared__ int s_last, s_flag, s_a, s_b, s_hit;
   __shared__ double s_sums[kSums];
-  __shared__ double s_part[8][kSums];
+  __shared__ ItemSumWord s_part_raw[8][kSums];
+  ItemSum (*s_part)[kSums] = reinterpret_cast<ItemSum (*)[kSums]>(s_part_raw);
   __shared__ double s_seed[12];
   // seed: every block that starts takes unseeded pairs until none is left
   for (;;) {
@@ -1760,21 +885,6 @@ int wave(K kernel, size_t smem) {
 }
 
 }  // namespace
-
-// association variant of these params (template bits kAGate | kAShoot)
-int assoc_variant(const KParams& P) { return (P.use_angle ? kAGate : 0) | (P.shoot_w > 0 ? kAShoot : 0); }
-
-// X(T, A) for the storage type and association variant of P
-#define KF_ASSOC_SWITCH(P, X)                                  \
-  do {                                                         \
-    const bool h_ = (P).precision == KF_FP16;                  \
-    switch (assoc_variant(P)) {                                \
-      case 0: if (h_) { X(__half, 0); } else { X(float, 0); } break; \
-      case 1: if (h_) { X(__half, 1); } else { X(float, 1); } break; \
-      case 2: if (h_) { X(__half, 2); } else { X(float, 2); } break; \
-      default: if (h_) { X(__half, 3); } else { X(float, 3); } break; \
-    }                                                          \
-  } while (0)
 
 void icp_grids(const KParams& P, int* g_assoc, int* g_reduce, int* g_sched) {
   const size_t sm = (size_t)P.bins * sizeof(unsigned), ss = sched_smem(P);
@@ -1912,8 +1022,9 @@ __global__ void __launch_bounds__(kBlock, 2) k_noalloc_reduce(unsigned char* scr
   for (int k = 0; k < kSums; ++k) sum[k] = 0.f;
   for (int i = begin + threadIdx.x; i < end; i += kBlock) {
     float p[3];
-    const int j = project(L, a.fv[3 * i], a.fv[3 * i + 1], a.fv[3 * i + 2], sxf, p);
+    const int j = project_any(L, a.fv[3 * i], a.fv[3 * i + 1], a.fv[3 * i + 2], sxf);
     if (j < 0) continue;
+    world_point(a.fv[3 * i], a.fv[3 * i + 1], a.fv[3 * i + 2], sxf, p);
     const float q[3] = {a.mv[3 * j], a.mv[3 * j + 1], a.mv[3 * j + 2]};
     const float n0 = a.mn[3 * j], n1 = a.mn[3 * j + 1], n2 = a.mn[3 * j + 2];
     // a model hole: any vertex or normal component non-finite, or a zero
@@ -1922,7 +1033,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_noalloc_reduce(unsigned char* scr
           isfinite(n2)) ||
         (n0 == 0.f && n1 == 0.f && n2 == 0.f))
       continue;
-    const int k = bin_of(p, q, a.P);
+    const int k = bin_any(p, q, a.P);
     if (k < a.klo || k > a.khi) continue;
     const float av[6] = {p[1] * n2 - p[2] * n1, p[2] * n0 - p[0] * n2, p[0] * n1 - p[1] * n0,
                          n0, n1, n2};

@@ -115,6 +115,12 @@ struct PairDesc {
                               // warp w of item li packs its records from place
                               // li * chunk + w * chunk / kBlockWarps
   unsigned* wcount;           // [items * kBlockWarps] records per item and warp
+  // team launch (null when the tracker's frames are too large for it): three
+  // rotating histograms, the leader's message and the half items' sums (packets
+  // of a value and its tag), all zero between launches but for the packets
+  unsigned* team_hist;        // [3 * team_hist_words(bins)]
+  unsigned long long* team_msg;   // [32]
+  unsigned long long* team_rows;  // [2 * items * 32]
   int* dbg_index;             // [iw*ih] inspection outputs (may be null)
   int* dbg_bin;
   int partial_cap;            // work-item partials the buffer holds
@@ -140,6 +146,15 @@ constexpr int kQHeaderWords = 256;
 constexpr int kMaxItemsPerLevel = 131071;  // 17-bit item field of a task
 constexpr int kMaxSchedPairs = 65535;      // 16-bit pair field
 
+// Team launch (kf_team.cu): words of one histogram (the bins to a multiple of
+// four, then the count of unmatched pixels), half items a worker block can
+// take, pairs of a launch.
+__host__ __device__ constexpr int team_hist_none(int bins) { return (bins + 3) / 4 * 4; }
+__host__ __device__ constexpr int team_hist_words(int bins) { return team_hist_none(bins) + 4; }
+constexpr int kTeamSlots = 8;
+constexpr int kTeamMaxItems = 1024;  // items of the largest frame
+constexpr int kTeamMaxPairs = 16;
+
 struct DescList {
   const PairDesc* d[kDescListMax];
   const float* depth[kDescListMax];  // level-0 raw depth of each pair (device)
@@ -153,7 +168,9 @@ struct KParams {
   int bins;
   float d_max32;
   float scale32;              // (float)(bins / d_max)
+  int tiny_bins;              // d_max or a bin's width at or below 2^-49
   double kappa;
+  int kappa_one;              // kappa == 1
   float cos_min32;
   int use_angle;
   int conv_window;
@@ -191,6 +208,26 @@ struct PairInput {
   int pad_;
 };
 
+struct PairOutput;
+
+// One pair of a team launch: its blocks are [first, first + 1 + workers), the
+// first its leader. tag: distinguishes this launch's packets from all earlier
+// ones (plus an iteration's number, below kTeamTags).
+struct TeamPair {
+  const PairDesc* d;
+  PairOutput* out;
+  unsigned tag;
+  int first, workers;
+};
+constexpr unsigned kTeamTags = 4096;  // > the iterations of an alignment + 1
+
+struct TeamArgs {
+  TeamPair pair[kTeamMaxPairs];
+  PairInput in[kTeamMaxPairs];
+  int n;
+  unsigned long long limit_ns;
+};
+
 struct PairOutput {
   double pose[16];
   kf_result res;
@@ -201,13 +238,15 @@ struct PairOutput {
 // the host reports it as KF_ERR_INTERNAL. Unchecked builds compile the guard
 // away and the access runs unconditionally.
 #ifdef KF_CHECKED
-__device__ void kf_fault(int code, long long a, long long b);
 #define KF_GUARD(cond, code, a, b) \
   if (!(cond)) {                   \
     kf_fault((code), (a), (b));    \
   } else
 #else
 #define KF_GUARD(cond, code, a, b)
+#endif
+#ifdef KF_CHECKED
+void checked_fault_team(long long out[3]);
 #endif
 // host side of checked builds: copies and clears the fault word (0 = none)
 void checked_fault(long long out[3]);
@@ -267,6 +306,10 @@ constexpr unsigned long long kSchedWaitLimitNs = 2000000000ull;  // 2 s
 cudaError_t launch_icp_sched(const PairDesc* const* descs, const PairInput* in, PairOutput* out,
                              int n, unsigned* queue, unsigned qmask, int grid,
                              unsigned long long wait_limit_ns, const KParams& P, cudaStream_t s);
+// the whole ICP of a few pairs, each by a team of resident blocks
+// (cooperative); team_blocks: blocks that can be resident at once
+int team_blocks(const KParams& P);
+cudaError_t launch_icp_team(const TeamArgs& args, int grid, const KParams& P, cudaStream_t s);
 cudaError_t launch_icp_finish(const PairDesc* const* descs, PairOutput* out, int n,
                               const KParams& P, cudaStream_t s);
 // inspection set-up of one pair: pose, level, band [klo, khi] and window
