@@ -156,7 +156,7 @@ KParams make_kparams(const kf_params* p) {
   k.bins = p->hist_bins;
   k.d_max32 = (float)p->d_max;
   k.scale32 = (float)((double)p->hist_bins / p->d_max);
-  k.tiny_bins = !(k.d_max32 > 0x1p-49f && k.scale32 < 0x1p49f);
+  k.tiny_bins = tiny_bins(k.d_max32, k.scale32);
   k.kappa = p->band_kappa;
   k.kappa_one = p->band_kappa == 1.0;
   k.cos_min32 = (float)p->cos_angle_min;

@@ -200,6 +200,9 @@ struct KParams {
   int shoot_w;                // normal-shooting window half-size (0: projective)
 };
 
+// d_max or a bin's width at or below 2^-49 (KParams::tiny_bins)
+inline bool tiny_bins(float d_max32, float scale32) { return !(d_max32 > 0x1p-49f && scale32 < 0x1p49f); }
+
 struct PairInput {
   double prior_R[9];
   double init[16];
