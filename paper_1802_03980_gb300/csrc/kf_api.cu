@@ -265,7 +265,6 @@ bool set_frame_levels(kf_tracker* t, const kf_intrinsics* K) {
     LevelMaps& L = t->h_desc.lv[l];
     L.fw = w;
     L.fh = h;
-    L.fps = frame_plane_stride(w, h);
     L.ffx = (float)fx;
     L.ffy = (float)fy;
     L.fcx = (float)cx;
@@ -543,23 +542,33 @@ float half_bits_to_float(uint16_t b) {
   return __half2float(__half(r));
 }
 
-// planes (x, y, z) of n elements of the map's storage type -> interleaved float
-// planes of `stride` elements (x, y, z) -> n interleaved xyz floats
-void planes_to_xyz(const std::vector<unsigned char>& buf, size_t n, size_t stride, size_t elem,
-                   float* out) {
-  for (size_t i = 0; i < n; ++i)
-    for (int c = 0; c < 3; ++c) {
-      const size_t k = c * stride + i;
-      float v;
-      if (elem == 4) {
-        memcpy(&v, buf.data() + 4 * k, 4);
-      } else {
-        uint16_t b;
-        memcpy(&b, buf.data() + 2 * k, 2);
-        v = half_bits_to_float(b);
-      }
-      out[3 * i + c] = v;
+// n pixels' vertices and normals (either may be null) from their records A and
+// B (see LevelMaps) as n interleaved xyz floats
+kf_status records_to_xyz(kf_tracker* t, const void* A, const void* B, size_t n, float* vertex, float* normal) {
+  std::vector<unsigned char> a(4 * n * t->elem), b(normal ? 2 * n * t->elem : 0);
+  KF_CK(t, cudaMemcpy(a.data(), A, a.size(), cudaMemcpyDeviceToHost));
+  if (normal) KF_CK(t, cudaMemcpy(b.data(), B, b.size(), cudaMemcpyDeviceToHost));
+  auto at = [&](const std::vector<unsigned char>& buf, size_t k) {
+    float v;
+    if (t->elem == 4) {
+      memcpy(&v, buf.data() + 4 * k, 4);
+    } else {
+      uint16_t h;
+      memcpy(&h, buf.data() + 2 * k, 2);
+      v = half_bits_to_float(h);
     }
+    return v;
+  };
+  for (size_t i = 0; i < n; ++i) {
+    if (vertex)
+      for (int c = 0; c < 3; ++c) vertex[3 * i + c] = at(a, 4 * i + c);
+    if (normal) {
+      normal[3 * i] = at(a, 4 * i + 3);
+      normal[3 * i + 1] = at(b, 2 * i);
+      normal[3 * i + 2] = at(b, 2 * i + 1);
+    }
+  }
+  return KF_OK;
 }
 
 }  // namespace
@@ -628,22 +637,19 @@ kf_status kf_track_create(const kf_params* p, int max_w, int max_h, void* cuda_s
     if (e != cudaSuccess) return bail(e);
     t->own_stream = true;
   }
-  // pixel buffers hold the largest level-0 plane rounded up, plus one
-  // alignment unit: bulk copies round a range's end up to 16 bytes
-  const size_t px0 = (size_t)frame_plane_stride(max_w, max_h) + kPlaneAlign;
+  const size_t px0 = (size_t)max_w * max_h;
   PairDesc& D = t->h_desc;
   D.levels = p->levels;
   if ((e = tmalloc(t, &t->d_depth_raw, px0 * sizeof(float))) != cudaSuccess) return bail(e);
   D.depth_raw = t->d_depth_raw;
   for (int l = 0; l < p->levels; ++l) {
     const size_t pl = (size_t)(max_w >> l) * (max_h >> l);
-    const size_t fpl = (size_t)frame_plane_stride(max_w >> l, max_h >> l) + kPlaneAlign;
     LevelMaps& L = D.lv[l];
     if ((e = tmalloc(t, &L.fdepth, pl * sizeof(float))) != cudaSuccess) return bail(e);
-    if ((e = tmalloc(t, &L.fV, 3 * fpl * t->elem)) != cudaSuccess) return bail(e);
-    if ((e = tmalloc(t, &L.fN, 3 * fpl * t->elem)) != cudaSuccess) return bail(e);
-    if ((e = tmalloc(t, &L.mV, 3 * pl * t->elem)) != cudaSuccess) return bail(e);
-    if ((e = tmalloc(t, &L.mN, 3 * pl * t->elem)) != cudaSuccess) return bail(e);
+    if ((e = tmalloc(t, &L.fA, 4 * pl * t->elem)) != cudaSuccess) return bail(e);
+    if ((e = tmalloc(t, &L.fB, 2 * pl * t->elem)) != cudaSuccess) return bail(e);
+    if ((e = tmalloc(t, &L.mA, 4 * pl * t->elem)) != cudaSuccess) return bail(e);
+    if ((e = tmalloc(t, &L.mB, 2 * pl * t->elem)) != cudaSuccess) return bail(e);
   }
   t->max_items = (int)(((size_t)max_w * max_h + kChunk - 1) / kChunk);
   if ((e = tmalloc(t, &t->d_state, sizeof(PairState))) != cudaSuccess) return bail(e);
@@ -1030,14 +1036,9 @@ kf_status kf_debug_frame_level(kf_tracker* t, int level, float* depth, float* ve
       dims[1] = L.fh;
     }
     if (depth) KF_CK(t, cudaMemcpy(depth, L.fdepth, n * sizeof(float), cudaMemcpyDeviceToHost));
-    std::vector<unsigned char> buf(3 * (size_t)L.fps * t->elem);
-    if (vertex) {
-      KF_CK(t, cudaMemcpy(buf.data(), L.fV, buf.size(), cudaMemcpyDeviceToHost));
-      planes_to_xyz(buf, n, L.fps, t->elem, vertex);
-    }
-    if (normal) {
-      KF_CK(t, cudaMemcpy(buf.data(), L.fN, buf.size(), cudaMemcpyDeviceToHost));
-      planes_to_xyz(buf, n, L.fps, t->elem, normal);
+    if (vertex || normal) {
+      const kf_status st = records_to_xyz(t, L.fA, L.fB, n, vertex, normal);
+      if (st != KF_OK) return st;
     }
     return KF_OK;
   } catch (...) {
@@ -1056,14 +1057,9 @@ kf_status kf_debug_model_level(kf_tracker* t, int level, float* vertex, float* n
       dims[0] = L.mw;
       dims[1] = L.mh;
     }
-    std::vector<unsigned char> buf(3 * n * t->elem);
-    if (vertex) {
-      KF_CK(t, cudaMemcpy(buf.data(), L.mV, buf.size(), cudaMemcpyDeviceToHost));
-      planes_to_xyz(buf, n, n, t->elem, vertex);
-    }
-    if (normal) {
-      KF_CK(t, cudaMemcpy(buf.data(), L.mN, buf.size(), cudaMemcpyDeviceToHost));
-      planes_to_xyz(buf, n, n, t->elem, normal);
+    if (vertex || normal) {
+      const kf_status st = records_to_xyz(t, L.mA, L.mB, n, vertex, normal);
+      if (st != KF_OK) return st;
     }
     return KF_OK;
   } catch (...) {

@@ -20,8 +20,7 @@ constexpr int kTx = 32, kTy = 8;
 
 __device__ __forceinline__ bool valid_depth(float z) { return isfinite(z) && z > 0.f; }
 
-// Model level l = level-0 model maps at pixels (x 2^l, y 2^l), converted to
-// planes; a pixel is a hole (NaN vertex and normal) when any component is
+// Model level l = level-0 model maps at pixels (x 2^l, y 2^l), as records; a pixel is a hole (NaN vertex and normal) when any component is
 // non-finite or the normal is all zero.
 template <class T>
 __global__ void __launch_bounds__(kTx* kTy) k_model_prep(const PairDesc* d, const float* Vin,
@@ -35,15 +34,9 @@ __global__ void __launch_bounds__(kTx* kTy) k_model_prep(const PairDesc* d, cons
   const bool ok = isfinite(vx) && isfinite(vy) && isfinite(vz) && isfinite(nx) && isfinite(ny) &&
                   isfinite(nz) && (nx != 0.f || ny != 0.f || nz != 0.f);
   const float nan = __int_as_float(0x7fc00000);
-  const int n = L.mw * L.mh, i = y * L.mw + x;
-  T* V = static_cast<T*>(L.mV);
-  T* N = static_cast<T*>(L.mN);
-  Store<T>::st(V, i, ok ? vx : nan);
-  Store<T>::st(V, n + i, ok ? vy : nan);
-  Store<T>::st(V, 2 * n + i, ok ? vz : nan);
-  Store<T>::st(N, i, ok ? nx : nan);
-  Store<T>::st(N, n + i, ok ? ny : nan);
-  Store<T>::st(N, 2 * n + i, ok ? nz : nan);
+  const int i = y * L.mw + x;
+  Store<T>::store_a(L.mA, i, ok ? make_float4(vx, vy, vz, nx) : make_float4(nan, nan, nan, nan));
+  Store<T>::store_b(L.mB, i, ok ? make_float2(ny, nz) : make_float2(nan, nan));
 }
 
 // ---------------------------------------------------------------------------
@@ -93,10 +86,7 @@ __device__ void write_maps(const LevelMaps& Lg, const float* Ds, int R, int ox, 
   // memory, which would force its fields to be reloaded for every pixel
   const LevelMaps L = Lg;
   // Ds: level depth region of R x R whose origin is level pixel (ox, oy)
-  const int n = L.fps;  // plane stride
   const float nan = __int_as_float(0x7fc00000);
-  T* V = static_cast<T*>(L.fV);
-  T* N = static_cast<T*>(L.fN);
   const float ifx = __fdiv_rn(1.f, L.ffx), ify = __fdiv_rn(1.f, L.ffy);
   const int tid = threadIdx.y * blockDim.x + threadIdx.x;
   for_region(tile, tile, tid, blockDim.x * blockDim.y, [&](int lx, int ly) {
@@ -140,14 +130,11 @@ __device__ void write_maps(const LevelMaps& Lg, const float* Ds, int R, int ox, 
       }
     }
     const int i = y * L.fw + x;
-    const bool keep = ok && nok;
     L.fdepth[i] = Ds[ly * R + lx];
-    Store<T>::st(V, i, keep ? v.x : nan);
-    Store<T>::st(V, n + i, keep ? v.y : nan);
-    Store<T>::st(V, 2 * n + i, keep ? v.z : nan);
-    Store<T>::st(N, i, nn.x);
-    Store<T>::st(N, n + i, nn.y);
-    Store<T>::st(N, 2 * n + i, nn.z);
+    // without a normal (which needs the vertex) both are NaN
+    if (!nok) v = nn;
+    Store<T>::store_a(L.fA, i, make_float4(v.x, v.y, v.z, nn.x));
+    Store<T>::store_b(L.fB, i, make_float2(nn.y, nn.z));
   });
 }
 
@@ -470,9 +457,6 @@ __global__ void __launch_bounds__(kTx * kTy) k_ii_normals(DescList list, IiGrid 
   }
   __syncthreads();
   // 5. four output pixels per thread
-  T* V = static_cast<T*>(L.fV);
-  T* N = static_cast<T*>(L.fN);
-  const int ps = L.fps;
   const float lscale = ldexpf(1.f, -l);
 #pragma unroll 1
   for (int part = 0; part < kIiRows / kTy; ++part) {
@@ -525,12 +509,8 @@ __global__ void __launch_bounds__(kTx * kTy) k_ii_normals(DescList list, IiGrid 
       }
     }
     const int i = y * W + x;
-    Store<T>::st(V, i, ok ? v.x : nan);
-    Store<T>::st(V, ps + i, ok ? v.y : nan);
-    Store<T>::st(V, 2 * ps + i, ok ? v.z : nan);
-    Store<T>::st(N, i, n[0]);
-    Store<T>::st(N, ps + i, n[1]);
-    Store<T>::st(N, 2 * ps + i, n[2]);
+    Store<T>::store_a(L.fA, i, ok ? make_float4(v.x, v.y, v.z, n[0]) : make_float4(nan, nan, nan, n[0]));
+    Store<T>::store_b(L.fB, i, make_float2(n[1], n[2]));
   }
 }
 

@@ -214,8 +214,9 @@ __device__ void assoc_items(const PairDesc* d, const LevelMaps& L, int first, in
   constexpr bool kGate = (kA & kAGate) != 0;
   const int fn = L.fw * L.fh;
   float sum[kSumRegs];
-  Verts<kU> va;
-  Batch<kGate, kU> sa;
+  constexpr int kN = kBatchU<kA>, kPixels = kN * kBlock;  // of a lane, of the block
+  Verts<kN> va;
+  Batch<kGate, kN> sa;
   const int warp = threadIdx.x >> 5;
   for (int li = first; li < first + run; ++li) {
     const int ib = li * chunk, ie = min(fn, ib + chunk);
@@ -224,17 +225,17 @@ __device__ void assoc_items(const PairDesc* d, const LevelMaps& L, int first, in
     const int rbase = ib + warp * (chunk / kBlockWarps);
     int wc = 0;
     zero_sums(sum);
-    // batches of the item; the last one may be partial (kBatch need not
+    // batches of the item; the last one may be partial (kPixels need not
     // divide the item)
-    for (int b0 = ib; b0 < ie; b0 += kBatch) {
-      const int e = min(ie, b0 + kBatch);
+    for (int b0 = ib; b0 < ie; b0 += kPixels) {
+      const int e = min(ie, b0 + kPixels);
       load_verts<T>(L, b0, e, threadIdx.x, va);
       associate_batch<T, kA, kPass>(L, b0, threadIdx.x, va, sxf, P, sa);
       {  // L2 hints for this warp's next batch (of this item or the next)
-        int nb0 = b0 + kBatch, ne = e + kBatch;
+        int nb0 = b0 + kPixels, ne = e + kPixels;
         if (nb0 >= ie) {
           nb0 = ie;
-          ne = li + 1 < first + run ? min(fn, ie + kBatch) : ie;
+          ne = li + 1 < first + run ? min(fn, ie + kPixels) : ie;
         }
         ne = min(ne, fn);
         // the match offset of the warp's first matched pixel (0: none)

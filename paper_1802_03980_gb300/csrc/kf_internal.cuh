@@ -46,27 +46,22 @@ constexpr int kMaxBins = 4096;
 constexpr int kMaxWindow = 8;
 constexpr int kDescListMax = 64;    // pairs per front-end launch
 
-// Maps of one pyramid level. Every map is stored as planes: x plane, then y,
-// then z. Model planes hold (mw * mh) elements each; frame planes are fps
-// elements apart, fw * fh rounded up to a multiple of kPlaneAlign, so that
-// every plane and every item of a plane starts on a 128-byte boundary (bulk
-// copies need 16) and a copy rounded up past the last pixel stays inside.
-constexpr int kPlaneAlign = 64;
-__host__ __device__ constexpr int frame_plane_stride(int w, int h) {
-  return (w * h + kPlaneAlign - 1) / kPlaneAlign * kPlaneAlign;
-}
+// Maps of one pyramid level: a pixel's vertex and normal as two records, A =
+// (v.x, v.y, v.z, n.x) and B = (n.y, n.z), in float32 (16 and 8 bytes) or
+// float16 (8 and 4). One wide load or store a record instead of one a
+// component: a gather of a model pixel is two instructions and addresses
+// instead of six, the front end's output three stores instead of seven, a
+// normal-shooting candidate one load instead of three.
 struct LevelMaps {
   int fw, fh;                 // frame level size
-  int fps;                    // frame plane stride (elements)
   int mw, mh;                 // model level size
   float ffx, ffy, fcx, fcy;   // frame level intrinsics (vertex map)
   float mfx, mfy, mcx, mcy;   // model level intrinsics (projection)
   float* fdepth;              // filtered depth, fw * fh
-  void* fV;                   // frame vertices, camera frame; NaN where the
-                              // vertex or its normal is invalid
-  void* fN;                   // frame normals, camera frame; NaN invalid
-  void* mV;                   // model vertices, world frame; NaN at holes
-  void* mN;                   // model normals, world frame
+  void* fA;                   // frame records, camera frame; vertex and normal NaN where
+  void* fB;                   // either is invalid
+  void* mA;                   // model records, world frame; NaN at holes
+  void* mB;
 };
 
 struct PairState {
@@ -257,12 +252,37 @@ void checked_fault(long long out[3]);
 // ---- storage-type helpers -------------------------------------------------
 template <class T> struct Store;
 template <> struct Store<float> {
-  static __device__ __forceinline__ float ld(const float* p, int i) { return __ldg(p + i); }
-  static __device__ __forceinline__ void st(float* p, int i, float v) { p[i] = v; }
+  using A = float4;
+  using B = float2;
+  static __device__ __forceinline__ float4 load_a(const void* p, int i) { return __ldg(static_cast<const float4*>(p) + i); }
+  static __device__ __forceinline__ float2 load_b(const void* p, int i) { return __ldg(static_cast<const float2*>(p) + i); }
+  static __device__ __forceinline__ void store_a(void* p, int i, float4 v) { static_cast<float4*>(p)[i] = v; }
+  static __device__ __forceinline__ void store_b(void* p, int i, float2 v) { static_cast<float2*>(p)[i] = v; }
 };
 template <> struct Store<__half> {
-  static __device__ __forceinline__ float ld(const __half* p, int i) { return __half2float(p[i]); }
-  static __device__ __forceinline__ void st(__half* p, int i, float v) { p[i] = __float2half_rn(v); }
+  using A = uint2;
+  using B = unsigned;
+  static __device__ __forceinline__ float2 pair(unsigned w) {
+    return __half22float2(*reinterpret_cast<const __half2*>(&w));
+  }
+  static __device__ __forceinline__ unsigned pack(float x, float y) {
+    const __half2 h = __floats2half2_rn(x, y);
+    return *reinterpret_cast<const unsigned*>(&h);
+  }
+  static __device__ __forceinline__ float4 load_a(const void* p, int i) {
+    const uint2 w = __ldg(static_cast<const uint2*>(p) + i);
+    const float2 a = pair(w.x), b = pair(w.y);
+    return make_float4(a.x, a.y, b.x, b.y);
+  }
+  static __device__ __forceinline__ float2 load_b(const void* p, int i) {
+    return pair(__ldg(static_cast<const unsigned*>(p) + i));
+  }
+  static __device__ __forceinline__ void store_a(void* p, int i, float4 v) {
+    static_cast<uint2*>(p)[i] = make_uint2(pack(v.x, v.y), pack(v.z, v.w));
+  }
+  static __device__ __forceinline__ void store_b(void* p, int i, float2 v) {
+    static_cast<unsigned*>(p)[i] = pack(v.x, v.y);
+  }
 };
 
 }  // namespace kf

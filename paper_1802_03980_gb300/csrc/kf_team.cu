@@ -169,9 +169,9 @@ __device__ __noinline__ void team_item(const PairDesc* d, const LevelMaps& maps,
   // eight pixels of a lane in flight where it has eight or more: one warp on
   // each scheduler has nothing else to hide its gathers behind
   if (chunk >= 8 * kBlock && !kShoots)
-    team_pass<T, kA, kPass, kShoots ? 4 : 8>(d, L, li, vw, chunk, sxf, P, sh_hist, lo, hi, sum, wc);
+    team_pass<T, kA, kPass, kShoots ? kBatchU<kA> : 8>(d, L, li, vw, chunk, sxf, P, sh_hist, lo, hi, sum, wc);
   else
-    team_pass<T, kA, kPass, 4>(d, L, li, vw, chunk, sxf, P, sh_hist, lo, hi, sum, wc);
+    team_pass<T, kA, kPass, kShoots ? kBatchU<kA> : 4>(d, L, li, vw, chunk, sxf, P, sh_hist, lo, hi, sum, wc);
   if constexpr (kPass != kPassHist) {
     const float r = warp_sums(sum);
     if ((threadIdx.x & 31) < kSums) row[threadIdx.x & 31] = r;
