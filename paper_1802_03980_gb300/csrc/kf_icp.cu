@@ -260,6 +260,179 @@ __device__ void assoc_items(const PairDesc* d, const LevelMaps& L, int first, in
   __syncthreads();
 }
 
+// ---------------------------------------------------------------------------
+// The scheduled kernel's association pass (projective, no gate): as
+// assoc_items, with the frame and model records passing through a ring in
+// shared memory. A thread copies its pixels' records into its own places
+// (cp.async), kAhead + 1 batches ahead for the frame and kAhead for the model,
+// so a gather is in flight while the batches before it are summed and holds no
+// registers meanwhile. What bounds the pass is the latency of a batch's
+// dependent loads (frame record, then the model pixel it projects to) against
+// the 16 to 24 warps an SM holds; with register gathers a warp spent 1850
+// cycles a pixel of its own at 43 % issue. Only a thread's own copies are waited for
+// (cp.async.wait_group): no barrier. The same pixels in the same order as
+// assoc_items: the same sums.
+// Measured on GB300, the whole alignment of a batch, register gathers -> ring:
+// 256 pairs 640x480 3.92 -> 3.55 ms, 64 mixed pairs float16 2.27 -> 2.03 ms, 32
+// pairs 0.85 -> 0.81 ms. Two pixels a batch: one pixel 4.2 ms (256 pairs), four
+// 3.74 (its registers); model records two or three batches ahead 3.53, 3.57; 24
+// warps on an SM 5.3 (spills).
+// ---------------------------------------------------------------------------
+#ifndef KF_RING_U
+#define KF_RING_U 2
+#endif
+constexpr int kRingU = KF_RING_U;  // pixels of a thread per batch
+static_assert(level_chunk(KF_MAX_LEVELS - 1) % (kRingU * kBlock) == 0, "a batch lies in one item");
+// bytes of the block's histogram, rounded up for what follows it
+__host__ __device__ __forceinline__ size_t hist_bytes(const KParams& P) {
+  return ((size_t)P.bins * sizeof(unsigned) + 15) / 16 * 16;
+}
+#ifndef KF_RING_AHEAD
+#define KF_RING_AHEAD 1
+#endif
+constexpr int kAhead = KF_RING_AHEAD;  // batches whose model records are under way
+template <class T>
+struct Ring {
+  typename Store<T>::A frame[kAhead + 2][kRingU][kBlock];
+  typename Store<T>::A model[kAhead + 1][kRingU][kBlock];
+  typename Store<T>::B normal[kAhead + 1][kRingU][kBlock];
+};
+
+template <class W>
+__device__ __forceinline__ void copy_async(W* dst, const W* src) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(dst);
+  if constexpr (sizeof(W) == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(src) : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(s), "l"(src), "n"(sizeof(W)) : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int kPending>
+__device__ __forceinline__ void copy_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(kPending) : "memory");
+}
+
+template <class T, int kPass>
+__device__ void assoc_ring(const PairDesc* d, const LevelMaps& L, int first, int run, int chunk,
+                           const float* sxf, const KParams& P, unsigned* sh_hist, Ring<T>* ring, int lo,
+                           int hi) {
+  using A = typename Store<T>::A;
+  using B = typename Store<T>::B;
+  constexpr int kN = kRingU, kPixels = kN * kBlock;
+  const int t = threadIdx.x, warp = t >> 5;
+  const int begin = first * chunk, end = min(L.fw * L.fh, begin + run * chunk);
+  const A* fA = static_cast<const A*>(L.fA);
+  const A* mA = static_cast<const A*>(L.mA);
+  const B* mB = static_cast<const B*>(L.mB);
+  auto fetch_frame = [&](int b0, int stage) {
+#pragma unroll
+    for (int u = 0; u < kN; ++u) {
+      const int i = b0 + t + u * kBlock;
+      if (i < end) copy_async(&ring->frame[stage][u][t], fA + i);
+    }
+    copy_commit();
+  };
+  // model pixels of the batches under way, oldest first
+  int j[kAhead + 1][kN];
+  // projects a batch whose frame records have come and sends for its model records
+  auto fetch_model = [&](int b0, int fstage, int mstage, int (&jj)[kN]) {
+    float xr[12];
+    load_xf<12>(sxf + 12, xr);
+    bool far = false;
+#pragma unroll
+    for (int u = 0; u < kN; ++u) {
+      const float4 v = Store<T>::value_a(ring->frame[fstage][u][t]);
+      jj[u] = project(L, v.x, v.y, v.z, xr, far);
+    }
+    if (far) {
+#pragma unroll
+      for (int u = 0; u < kN; ++u) {
+        const float4 v = Store<T>::value_a(ring->frame[fstage][u][t]);
+        jj[u] = project_far(v.x, v.y, v.z, L.mw, L.mh, L.mfx, L.mfy, L.mcx, L.mcy, sxf);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kN; ++u) {
+      if (b0 + t + u * kBlock >= end) jj[u] = -1;
+      if (jj[u] >= 0) {
+        copy_async(&ring->model[mstage][u][t], mA + jj[u]);
+        if constexpr (kPass != kPassHist) copy_async(&ring->normal[mstage][u][t], mB + jj[u]);
+      }
+    }
+    copy_commit();
+  };
+  // the loop's order of groups from the start on: the frame of batch k + 1, then
+  // the model of batch k
+  fetch_frame(begin, 0);
+#pragma unroll
+  for (int k = 0; k < kAhead; ++k) {
+    fetch_frame(begin + (k + 1) * kPixels, k + 1);
+    if (k == 0) copy_wait<1>();
+    else copy_wait<2>();
+    fetch_model(begin + k * kPixels, k, k, j[k]);
+  }
+  float sum[kSumRegs];
+  zero_sums(sum);
+  int wc = 0, fs = 0, ms = 0;  // the ring places of the batch being summed
+  for (int b0 = begin; b0 < end; b0 += kPixels) {
+    // the batch kAhead later: its frame records have come (one model group
+    // stands behind them); the frame records after them take the free place
+    copy_wait<1>();
+    const int fl = fs + kAhead < kAhead + 2 ? fs + kAhead : fs - 2;
+    const int ff = fl + 1 < kAhead + 2 ? fl + 1 : 0;
+    fetch_frame(b0 + (kAhead + 1) * kPixels, ff);
+    fetch_model(b0 + kAhead * kPixels, fl, ms > 0 ? ms - 1 : kAhead, j[kAhead]);
+    copy_wait<2 * kAhead>();  // this batch's model records
+    Batch<false, kN> cur;
+    {
+      float xw[12];
+      load_xf<12>(sxf, xw);
+#pragma unroll
+      for (int u = 0; u < kN; ++u) {
+        const float4 v = Store<T>::value_a(ring->frame[fs][u][t]);
+        world_point(v.x, v.y, v.z, xw, cur.p[u]);
+        cur.j[u] = j[0][u];
+        const float4 q = Store<T>::value_a(ring->model[ms][u][t]);
+        cur.q[u][0] = q.x;
+        cur.q[u][1] = q.y;
+        cur.q[u][2] = q.z;
+        cur.nq[u][0] = q.w;
+        if constexpr (kPass != kPassHist) {
+          const float2 n = Store<T>::value_b(ring->normal[ms][u][t]);
+          cur.nq[u][1] = n.x;
+          cur.nq[u][2] = n.y;
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k)
+#pragma unroll
+      for (int u = 0; u < kN; ++u) j[k][u] = j[k + 1][u];
+    fs = fs + 1 < kAhead + 2 ? fs + 1 : 0;
+    ms = ms < kAhead ? ms + 1 : 0;
+    const int li = b0 / chunk;
+    const int rbase = li * chunk + warp * (chunk / kBlockWarps);
+    finish_batch<0, kPass, 0>(d, b0, end, t, cur, sxf, P, sh_hist, lo, hi, sum, rbase, wc);
+    const int after = b0 + kPixels;
+    if (after >= end || after % chunk == 0) {  // the item's last batch
+      if constexpr (kPass == kPassSplit) {
+        if ((t & 31) == 0) {
+          KF_GUARD(li < d->partial_cap, 7, li, d->partial_cap)
+          d->wcount[li * kBlockWarps + warp] = wc;
+        }
+        wc = 0;
+      }
+      if constexpr (kPass != kPassHist) {
+        KF_GUARD(li < d->partial_cap, 1, li, d->partial_cap)
+        write_row(d, li, kPass == kPassBand, sum);
+        zero_sums(sum);
+      }
+    }
+  }
+  copy_wait<0>();
+  __syncthreads();
+}
+
 __device__ __forceinline__ int record_count(const PairDesc* d, int li) {
   return li < d->partial_cap ? (int)__ldcg(d->wcount + li * kBlockWarps + (threadIdx.x >> 5)) : 0;
 }
@@ -747,7 +920,9 @@ __global__ void __launch_bounds__(kBlock, KF_SCHED_MINB) k_icp_sched(const PairD
                                                                      unsigned qmask,
                                                                      unsigned long long limit_ns,
                                                                      KParams P) {
-  extern __shared__ unsigned sh_hist[];
+  extern __shared__ __align__(16) unsigned char sh_raw[];
+  unsigned* sh_hist = reinterpret_cast<unsigned*>(sh_raw);
+  [[maybe_unused]] Ring<T>* ring = reinterpret_cast<Ring<T>*>(sh_raw + hist_bytes(P));
   __shared__ __align__(16) float sxf[24];  // 16-byte vector loads (load_xf)
   __shared__ unsigned long long s_word;
   __shared__ int s_last, s_flag, s_a, s_b, s_hit;
@@ -795,10 +970,16 @@ __global__ void __launch_bounds__(kBlock, KF_SCHED_MINB) k_icp_sched(const PairD
       }
       for (int b = threadIdx.x; b < P.bins; b += kBlock) sh_hist[b] = 0u;
       __syncthreads();
-      if (s_a >= 0)
+      if constexpr (kA == 0) {
+        if (s_a >= 0)
+          assoc_ring<T, kPassSplit>(d, L, first, run, chunk, sxf, P, sh_hist, ring, s_a, s_b);
+        else
+          assoc_ring<T, kPassHist>(d, L, first, run, chunk, sxf, P, sh_hist, ring, 0, 0);
+      } else if (s_a >= 0) {
         assoc_items<T, kA, kPassSplit, 0>(d, L, first, run, chunk, sxf, P, sh_hist, s_a, s_b);
-      else
+      } else {
         assoc_items<T, kA, kPassHist, 0>(d, L, first, run, chunk, sxf, P, sh_hist, 0, 0);
+      }
       for (int b = threadIdx.x; b < P.bins; b += kBlock) {
         const unsigned c = sh_hist[b];
         if (c) atomicAdd(d->hist + b, c);
@@ -851,7 +1032,10 @@ __global__ void __launch_bounds__(kBlock, KF_SCHED_MINB) k_icp_sched(const PairD
       } else {
         // re-association with the band known (items in increasing order; the
         // partials do not depend on it)
-        assoc_items<T, kA, kPassBand, 0>(d, L, first, run, chunk, sxf, P, nullptr, s_a, s_b);
+        if constexpr (kA == 0)
+          assoc_ring<T, kPassBand>(d, L, first, run, chunk, sxf, P, nullptr, ring, s_a, s_b);
+        else
+          assoc_items<T, kA, kPassBand, 0>(d, L, first, run, chunk, sxf, P, nullptr, s_a, s_b);
       }
       __threadfence();
       __syncthreads();
@@ -872,8 +1056,9 @@ __global__ void __launch_bounds__(kBlock, KF_SCHED_MINB) k_icp_sched(const PairD
   }
 }
 
-// the block's histogram
-size_t sched_smem(const KParams& P) { return (size_t)P.bins * sizeof(unsigned); }
+// the block's histogram, and the ring of the variants that have one
+template <class T, int kA>
+size_t sched_smem(const KParams& P) { return hist_bytes(P) + (kA == 0 ? sizeof(Ring<T>) : 0); }
 
 template <class K>
 int wave(K kernel, size_t smem) {
@@ -888,11 +1073,11 @@ int wave(K kernel, size_t smem) {
 }  // namespace
 
 void icp_grids(const KParams& P, int* g_assoc, int* g_reduce, int* g_sched) {
-  const size_t sm = (size_t)P.bins * sizeof(unsigned), ss = sched_smem(P);
+  const size_t sm = (size_t)P.bins * sizeof(unsigned);
 #define KF_X(T, A)                                 \
   *g_assoc = wave(k_assoc_hist<T, A>, sm);         \
   *g_reduce = wave(k_reduce_solve<T, A>, 0);       \
-  *g_sched = wave(k_icp_sched<T, A>, ss)
+  *g_sched = wave(k_icp_sched<T, A>, sched_smem<T, A>(P))
   KF_ASSOC_SWITCH(P, KF_X);
 #undef KF_X
   // one partition of the items for both passes
@@ -902,10 +1087,9 @@ void icp_grids(const KParams& P, int* g_assoc, int* g_reduce, int* g_sched) {
 cudaError_t launch_icp_sched(const PairDesc* const* descs, const PairInput* in, PairOutput* out,
                              int n, unsigned* queue, unsigned qmask, int grid,
                              unsigned long long wait_limit_ns, const KParams& P, cudaStream_t s) {
-  const size_t sm = sched_smem(P);
   unsigned long long* slots = reinterpret_cast<unsigned long long*>(queue + kQHeaderWords);
 #define KF_X(T, A) \
-  k_icp_sched<T, A><<<grid, kBlock, sm, s>>>(descs, in, out, n, queue, slots, qmask, wait_limit_ns, P)
+  k_icp_sched<T, A><<<grid, kBlock, sched_smem<T, A>(P), s>>>(descs, in, out, n, queue, slots, qmask, wait_limit_ns, P)
   KF_ASSOC_SWITCH(P, KF_X);
 #undef KF_X
   return cudaGetLastError();
@@ -1043,7 +1227,8 @@ __global__ void __launch_bounds__(kBlock) k_noalloc_reduce(unsigned char* scratc
 #pragma unroll
     for (int u = 0; u < kNoAllocFly; ++u) {
       if constexpr (kShort) {
-        j[u] = project(L, v[u][0], v[u][1], v[u][2], sxf, p[u], far);
+        world_point(v[u][0], v[u][1], v[u][2], sxf, p[u]);
+        j[u] = project(L, v[u][0], v[u][1], v[u][2], sxf + 12, far);
       } else {
         world_point(v[u][0], v[u][1], v[u][2], sxf, p[u]);
         j[u] = project_any(L, v[u][0], v[u][1], v[u][2], sxf);

@@ -254,6 +254,8 @@ template <class T> struct Store;
 template <> struct Store<float> {
   using A = float4;
   using B = float2;
+  static __device__ __forceinline__ float4 value_a(float4 w) { return w; }
+  static __device__ __forceinline__ float2 value_b(float2 w) { return w; }
   static __device__ __forceinline__ float4 load_a(const void* p, int i) { return __ldg(static_cast<const float4*>(p) + i); }
   static __device__ __forceinline__ float2 load_b(const void* p, int i) { return __ldg(static_cast<const float2*>(p) + i); }
   static __device__ __forceinline__ void store_a(void* p, int i, float4 v) { static_cast<float4*>(p)[i] = v; }
@@ -269,13 +271,16 @@ template <> struct Store<__half> {
     const __half2 h = __floats2half2_rn(x, y);
     return *reinterpret_cast<const unsigned*>(&h);
   }
-  static __device__ __forceinline__ float4 load_a(const void* p, int i) {
-    const uint2 w = __ldg(static_cast<const uint2*>(p) + i);
+  static __device__ __forceinline__ float4 value_a(uint2 w) {
     const float2 a = pair(w.x), b = pair(w.y);
     return make_float4(a.x, a.y, b.x, b.y);
   }
+  static __device__ __forceinline__ float2 value_b(unsigned w) { return pair(w); }
+  static __device__ __forceinline__ float4 load_a(const void* p, int i) {
+    return value_a(__ldg(static_cast<const uint2*>(p) + i));
+  }
   static __device__ __forceinline__ float2 load_b(const void* p, int i) {
-    return pair(__ldg(static_cast<const unsigned*>(p) + i));
+    return value_b(__ldg(static_cast<const unsigned*>(p) + i));
   }
   static __device__ __forceinline__ void store_a(void* p, int i, float4 v) {
     static_cast<uint2*>(p)[i] = make_uint2(pack(v.x, v.y), pack(v.z, v.w));
