@@ -184,6 +184,7 @@ KParams make_kparams(const kf_params* p) {
     const int dy = i / wd - r, dx = i % wd - r;
     k.bil_sw2[i] = (float)(-(double)(dx * dx + dy * dy) * log2e /
                            (2.0 * p->bilateral_sigma_s * p->bilateral_sigma_s));
+    k.bil_nsw[dx * dx + dy * dy] = -k.bil_sw2[i];
   }
   k.bil_c2 = (float)(log2e / (2.0 * p->bilateral_sigma_r * p->bilateral_sigma_r));
   k.bil_k = (float)std::sqrt(log2e / (2.0 * p->bilateral_sigma_r * p->bilateral_sigma_r));

@@ -10,7 +10,7 @@ namespace {
 constexpr int kTx = 32, kTy = 8;
 // resident front-end blocks per SM the register budget is sized for
 #ifndef KF_FE_MINB
-#define KF_FE_MINB 7
+#define KF_FE_MINB 6
 #endif
 // bilateral filter: 1 two vertically adjacent pixels per thread step with
 // packed FP32x2 arithmetic; 0 one pixel per step (the same bits either way)
@@ -80,62 +80,70 @@ __device__ __forceinline__ void for_region(int w, int h, int tid, int nthr, F f)
   }
 }
 
-template <class T>
-__device__ void write_maps(const LevelMaps& Lg, const float* Ds, int R, int ox, int oy, int tile) {
+// The vertex of the pixel with (u - c) = (ux, uy) and depth z, and whether it
+// has one: x = (u_c z) / f as (u_c z) (1 / f), each product rounded.
+__device__ __forceinline__ bool back_project(float ux, float uy, float ifx, float ify, float z, float3& v) {
+  v.x = __fmul_rn(__fmul_rn(ux, z), ifx);
+  v.y = __fmul_rn(__fmul_rn(uy, z), ify);
+  v.z = z;
+  return z > 0.f;
+}
+
+// Maps of a level's tile x tile pixels from (ox, oy) on. A thread takes kRows
+// pixels below one another: the column's coordinates are formed once, and a
+// pixel's lower neighbour is the next pixel. Ds: level depth region of R x R
+// whose origin is level pixel (ox, oy).
+template <class T, int kTileL, int kRows>
+__device__ __forceinline__ void write_maps(const LevelMaps& Lg, const float* Ds, int R, int ox, int oy) {
   // a local copy: the map stores below could alias the descriptor in global
   // memory, which would force its fields to be reloaded for every pixel
   const LevelMaps L = Lg;
-  // Ds: level depth region of R x R whose origin is level pixel (ox, oy)
   const float nan = __int_as_float(0x7fc00000);
   const float ifx = __fdiv_rn(1.f, L.ffx), ify = __fdiv_rn(1.f, L.ffy);
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-  for_region(tile, tile, tid, blockDim.x * blockDim.y, [&](int lx, int ly) {
-    const int x = ox + lx, y = oy + ly;
-    if (x >= L.fw || y >= L.fh) return;
-    // (u - c) for the pixel and its right / lower neighbour; (float)(x + 1)
-    // is (float)x + 1 exactly for image coordinates
-    const float fx0 = (float)x, fy0 = (float)y;
-    const float ux0 = __fsub_rn(fx0, L.fcx), ux1 = __fsub_rn(fx0 + 1.f, L.fcx);
-    const float uy0 = __fsub_rn(fy0, L.fcy), uy1 = __fsub_rn(fy0 + 1.f, L.fcy);
-    // vertex: x = (u_c z) / f as (u_c z) (1 / f), each product rounded
-    auto bp = [&](float ux, float uy, int sx, int sy, float3& v) -> bool {
-      const float z = Ds[sy * R + sx];
-      if (!(z > 0.f)) return false;
-      v.x = __fmul_rn(__fmul_rn(ux, z), ifx);
-      v.y = __fmul_rn(__fmul_rn(uy, z), ify);
-      v.z = z;
-      return true;
-    };
-    float3 v, v10, v01, nn = make_float3(nan, nan, nan);
-    const bool ok = bp(ux0, uy0, lx, ly, v);
-    bool nok = false;
-    if (ok && x + 1 < L.fw && y + 1 < L.fh && bp(ux1, uy0, lx + 1, ly, v10) &&
-        bp(ux0, uy1, lx, ly + 1, v01)) {
-      // the decisions (a normal exists; it faces the camera) are float32 with
-      // every operation rounded in this order, no contraction: a = v10 - v,
-      // b = v01 - v; c = a x b, products rounded, then the difference;
-      // l2 = (cx cx + cy cy) + cz cz: a normal iff finite and > 0;
-      // s = (cx vx + cy vy) + cz vz > 0 flips it (decided before normalising)
-      const float ax = __fsub_rn(v10.x, v.x), ay = __fsub_rn(v10.y, v.y), az = __fsub_rn(v10.z, v.z);
-      const float bx = __fsub_rn(v01.x, v.x), by = __fsub_rn(v01.y, v.y), bz = __fsub_rn(v01.z, v.z);
-      const float cx = __fsub_rn(__fmul_rn(ay, bz), __fmul_rn(az, by));
-      const float cy = __fsub_rn(__fmul_rn(az, bx), __fmul_rn(ax, bz));
-      const float cz = __fsub_rn(__fmul_rn(ax, by), __fmul_rn(ay, bx));
-      const float len2 = __fadd_rn(__fadd_rn(__fmul_rn(cx, cx), __fmul_rn(cy, cy)), __fmul_rn(cz, cz));
-      if (len2 > 0.f && isfinite(len2)) {
-        const float sd = __fadd_rn(__fadd_rn(__fmul_rn(cx, v.x), __fmul_rn(cy, v.y)), __fmul_rn(cz, v.z));
-        const float inv = sd > 0.f ? -rsqrtf(len2) : rsqrtf(len2);
-        nn = make_float3(cx * inv, cy * inv, cz * inv);
-        nok = true;
-      }
-    }
+  const int tid = threadIdx.y * kTx + threadIdx.x;
+  if (tid >= kTileL * kTileL / kRows) return;
+  const int lx = tid % kTileL, ly0 = tid / kTileL * kRows;
+  const int x = ox + lx;
+  if (x >= L.fw) return;
+  // (float)(x + 1) is (float)x + 1 exactly for image coordinates
+  const float fx0 = (float)x, fy0 = (float)(oy + ly0);
+  const float ux0 = __fsub_rn(fx0, L.fcx), ux1 = __fsub_rn(fx0 + 1.f, L.fcx);
+  const float* D = Ds + ly0 * R + lx;
+  const bool right = x + 1 < L.fw;
+  float3 v;
+  float uy = __fsub_rn(fy0, L.fcy);
+  bool ok = back_project(ux0, uy, ifx, ify, D[0], v);
+#pragma unroll
+  for (int r = 0; r < kRows; ++r, D += R) {
+    const int y = oy + ly0 + r;
+    if (y >= L.fh) return;
+    const float uy1 = __fsub_rn(fy0 + (float)(r + 1), L.fcy);
+    float3 v10, v01;
+    const bool ok10 = back_project(ux1, uy, ifx, ify, D[1], v10);
+    const bool ok01 = back_project(ux0, uy1, ifx, ify, D[R], v01);
+    // the decisions (a normal exists; it faces the camera) are float32 with
+    // every operation rounded in this order, no contraction: a = v10 - v,
+    // b = v01 - v; c = a x b, products rounded, then the difference;
+    // l2 = (cx cx + cy cy) + cz cz: a normal iff finite and > 0;
+    // s = (cx vx + cy vy) + cz vz > 0 flips it (decided before normalising)
+    const float ax = __fsub_rn(v10.x, v.x), ay = __fsub_rn(v10.y, v.y), az = __fsub_rn(v10.z, v.z);
+    const float bx = __fsub_rn(v01.x, v.x), by = __fsub_rn(v01.y, v.y), bz = __fsub_rn(v01.z, v.z);
+    const float cx = __fsub_rn(__fmul_rn(ay, bz), __fmul_rn(az, by));
+    const float cy = __fsub_rn(__fmul_rn(az, bx), __fmul_rn(ax, bz));
+    const float cz = __fsub_rn(__fmul_rn(ax, by), __fmul_rn(ay, bx));
+    const float len2 = __fadd_rn(__fadd_rn(__fmul_rn(cx, cx), __fmul_rn(cy, cy)), __fmul_rn(cz, cz));
+    const float sd = __fadd_rn(__fadd_rn(__fmul_rn(cx, v.x), __fmul_rn(cy, v.y)), __fmul_rn(cz, v.z));
+    const bool nok = ok && ok10 && ok01 && right && y + 1 < L.fh && len2 > 0.f && len2 < __int_as_float(0x7f800000);
+    const float len = rsqrtf(len2), inv = sd > 0.f ? -len : len;
     const int i = y * L.fw + x;
-    L.fdepth[i] = Ds[ly * R + lx];
+    L.fdepth[i] = D[0];
     // without a normal (which needs the vertex) both are NaN
-    if (!nok) v = nn;
-    Store<T>::store_a(L.fA, i, make_float4(v.x, v.y, v.z, nn.x));
-    Store<T>::store_b(L.fB, i, make_float2(nn.y, nn.z));
-  });
+    Store<T>::store_a(L.fA, i, nok ? make_float4(v.x, v.y, v.z, cx * inv) : make_float4(nan, nan, nan, nan));
+    Store<T>::store_b(L.fB, i, nok ? make_float2(cy * inv, cz * inv) : make_float2(nan, nan));
+    v = v01;
+    ok = ok01;
+    uy = uy1;
+  }
 }
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -167,9 +175,11 @@ __device__ __forceinline__ float2 bilateral_pair(const float2* s_pair, int RR, i
     for (int dx = -R; dx <= R; ++dx) {
       const float2 zn = s_pair[(cy + dy) * RR + cx + dx];
       const float2 sd = __ffma2_rn(zn, k2, mkz);
-      const float sw = P.bil_sw2[(dy + R) * (2 * R + 1) + dx + R];
-      const float2 e = __ffma2_rn(make_float2(-sd.x, -sd.y), sd, make_float2(sw, sw));
-      const float2 wt = make_float2(ex2_approx(e.x), ex2_approx(e.y));
+      // the exponent's negative, sd^2 - sw: a packed operation has no free sign,
+      // the exponential's operand has; one weight per distance, held in registers
+      const float nsw = P.bil_nsw[dx * dx + dy * dy];
+      const float2 e = __ffma2_rn(sd, sd, make_float2(nsw, nsw));
+      const float2 wt = make_float2(ex2_approx(-e.x), ex2_approx(-e.y));
       num = __ffma2_rn(wt, zn, num);
       den = __fadd2_rn(den, wt);
     }
@@ -296,8 +306,10 @@ __global__ void __launch_bounds__(kTx* kTy, KF_FE_MINB) k_frontend_fused(DescLis
     });
     __syncthreads();
   }
-  for (int l = 0; l < levels; ++l)
-    write_maps<T>(d->lv[l], lev[l], R0 >> l, X0 >> l, Y0 >> l, kTile >> l);
+  write_maps<T, kTile, 4>(d->lv[0], s_d0, R0, X0, Y0);
+  if (levels > 1) write_maps<T, kTile / 2, 1>(d->lv[1], s_d1, R0 >> 1, X0 >> 1, Y0 >> 1);
+  if (levels > 2) write_maps<T, kTile / 4, 1>(d->lv[2], s_d2, R0 >> 2, X0 >> 2, Y0 >> 2);
+  if (levels > 3) write_maps<T, kTile / 8, 1>(d->lv[3], s_d3, R0 >> 3, X0 >> 3, Y0 >> 3);
 }
 
 dim3 grid_for(int w, int h, int n) { return dim3((w + kTx - 1) / kTx, (h + kTy - 1) / kTy, n); }
