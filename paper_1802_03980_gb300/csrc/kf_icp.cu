@@ -121,10 +121,14 @@ __device__ __noinline__ int median_and_band(const PairDesc* d, PairState* st, co
 __device__ __noinline__ int solve_update_warp(const PairDesc* d, PairState* st, const double* S,
                                                int level, const KParams& P, int passes,
                                                const PairPre& pre) {
-  double Tc[3];
+  double Tc[3], Tmc[3], Tmt[3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) Tc[k] = __ldcg(&st->T[4 * k + (threadIdx.x & 3)]);
-  return solve_update(d, st, S, level, P, passes, pre, Tc, [](const Solved&, int, int, int) {});
+  load_tm(d->Tm, Tmc, Tmt);
+  const NextStep next = next_step(pre, level, P);
+  const double lam2c = lane_of(2.0 * pre.lambda_c, 0);
+  return solve_update(d, st, S, level, P, passes, pre, next, solve_lane(), lam2c, Tc, Tmc, Tmt,
+                      [](const Solved&, int, int, int) {});
 }
 
 // ---------------------------------------------------------------------------

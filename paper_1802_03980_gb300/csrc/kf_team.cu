@@ -21,7 +21,8 @@
 // the leader clears one once its iteration's sums have all come, two
 // iterations before it is used again.
 //
-// A half item is four of the eight warps of an item (0 2 4 6 or 1 3 5 7): the
+// A half item is four of the eight warps of an item (0 2 4 6 or 1 3 5 7), each
+// shared by two warps here (team_batch): the
 // rows, their halving within an item and the order over items are those
 // of the queue's launch, so the two give the same bits, and 150 blocks share a
 // 640x480 frame, one on an SM. A worker's frame and model pixels stay in its
@@ -43,8 +44,8 @@ void checked_fault_team(long long out[3]) { take_fault(out); }
 
 namespace {
 
-constexpr int kTeamWarps = 4;
-constexpr int kTeamBlock = 32 * kTeamWarps;
+constexpr int kTeamWarps = 4;            // item warps of a half item
+constexpr int kTeamBlock = 2 * 32 * kTeamWarps;  // two warps (parts) for each
 constexpr int kPollCheck = 64;  // polls between two looks at the clock
 
 __device__ __forceinline__ void packet_store(unsigned long long* p, unsigned v, unsigned tag) {
@@ -137,53 +138,17 @@ __device__ bool warp_median(const unsigned* hist, int bins, unsigned pixels,
   return true;
 }
 
-// An association pass of one warp of an item (virtual warp vw of the item's
-// eight): batches of kN pixels a lane, the same pixels in the same order as
-// assoc_items gives that warp.
-template <class T, int kA, int kPass, int kN>
-__device__ __forceinline__ void team_pass(const PairDesc* d, const LevelMaps& L, int li, int vw,
-                                          int chunk, const float* sxf, const KParams& P,
-                                          unsigned* sh_hist, int lo, int hi, float* sum, int& wc) {
-  const int t = vw * 32 + (threadIdx.x & 31);
-  const int ib = li * chunk, ie = min(L.fw * L.fh, ib + chunk);
-  const int rbase = ib + vw * (chunk / kBlockWarps);
-  Verts<kN> v;
-  Batch<(kA & kAGate) != 0, kN> b;
-  for (int b0 = ib; b0 < ie; b0 += kN * kBlock) {
-    const int e = min(ie, b0 + kN * kBlock);
-    load_verts<T>(L, b0, e, t, v);
-    associate_batch<T, kA, kPass>(L, b0, t, v, sxf, P, b);
-    finish_batch<kA, kPass, 0>(d, b0, e, t, b, sxf, P, sh_hist, lo, hi, sum, rbase, wc);
-  }
-}
-
-template <class T, int kA, int kPass>
-__device__ __noinline__ void team_item(const PairDesc* d, const LevelMaps& maps, int li, int vw, int chunk,
-                                       const float* sxf, const KParams& P, unsigned* sh_hist, int lo,
-                                       int hi, float* row, int* count) {
-  constexpr bool kShoots = (kA & kAShoot) != 0;
-  const LevelMaps L = maps;  // in registers: the caller's copy lies in its stack frame
-  float sum[kSumRegs];
-  zero_sums(sum);
-  int wc = 0;
-  // eight pixels of a lane in flight where it has eight or more: one warp on
-  // each scheduler has nothing else to hide its gathers behind
-  if (chunk >= 8 * kBlock && !kShoots)
-    team_pass<T, kA, kPass, kShoots ? kBatchU<kA> : 8>(d, L, li, vw, chunk, sxf, P, sh_hist, lo, hi, sum, wc);
-  else
-    team_pass<T, kA, kPass, kShoots ? kBatchU<kA> : 4>(d, L, li, vw, chunk, sxf, P, sh_hist, lo, hi, sum, wc);
-  if constexpr (kPass != kPassHist) {
-    const float r = warp_sums(sum);
-    if ((threadIdx.x & 31) < kSums) row[threadIdx.x & 31] = r;
-  }
-  *count = wc;
+// Barrier of the two warps (parts) of one item warp.
+__device__ __forceinline__ void parts_sync(int lw) {
+  asm volatile("bar.sync %0, 64;" ::"r"(1 + lw) : "memory");
 }
 
 struct TeamShared {
   float xf[24];  // first: 16-byte vector loads (load_xf)
+  float hand[2][kTeamWarps][kSumRegs][32];  // part 0's sums per lane, for part 1 (by slot parity)
   float row_a[kTeamSlots][kTeamWarps][32];
   float row[2][kTeamWarps][32];
-  int count[kTeamSlots][kTeamWarps];
+  int count[kTeamSlots][kTeamWarps][2];  // records of each part
   double T[12];
   ItemSumWord part[kBlockWarps][kSums];
   double sums[kSums + 3];
@@ -191,6 +156,109 @@ struct TeamShared {
   int N, kmed, klo, khi, hit, stop;
   unsigned matched;
   int abort;
+};
+
+// An association pass of one warp (virtual warp vw of item li's eight), by two
+// warps: a lane's pixels, in the order assoc_items gives that warp, are cut in
+// two, part 0 takes the first half and part 1 the second. Each looks up, counts
+// and forms the rows of its kN pixels at the same time; only the additions stay
+// in order: part 0 hands its lanes' sums to part 1, which goes on from them and
+// writes the warp's row. Part 1's records start half a region on (fix_place).
+// Alone on its scheduler a warp took 5.9 us for the 16 pixels a lane has at level
+// 0 (640x480), two take 3.6 us.
+template <class T, int kA, int kPass, int kN>
+__device__ __forceinline__ void team_batch(const PairDesc* d, const LevelMaps& L, int li, int vw, int lw,
+                                           int part, int chunk, const KParams& P, TeamShared& sh, int s,
+                                           unsigned* sh_hist, int lo, int hi, float* row) {
+  const int lane = threadIdx.x & 31, t = vw * 32 + lane;
+  const int ib = li * chunk, b0 = ib + part * kN * kBlock;
+  const int e = min(min(L.fw * L.fh, ib + chunk), b0 + kN * kBlock);
+  Verts<kN> v;
+  Batch<(kA & kAGate) != 0, kN> b;
+  int bin[kN];
+  load_verts<T>(L, b0, e, t, v);
+  associate_batch<T, kA, kPass>(L, b0, t, v, sh.xf, P, b);
+  finish_bins<kA, kPass, 0, kN>(d, b0, e, t, b, sh.xf, P, sh_hist, bin);
+  if constexpr (kPass != kPassHist) {
+    float sum[kSumRegs];
+    float (*hand)[32] = sh.hand[s & 1][lw];
+    int wc = 0;
+    const int rbase = ib + vw * (chunk / kBlockWarps) + part * (chunk / kBlockWarps / 2);
+    if (part == 0) {
+      zero_sums(sum);
+      finish_rows<kA, kPass, kN>(d, b, bin, lo, hi, sum, rbase, wc);
+#pragma unroll
+      for (int k = 0; k < kSumRegs; ++k) hand[k][lane] = sum[k];
+      parts_sync(lw);
+    } else {
+      parts_sync(lw);
+#pragma unroll
+      for (int k = 0; k < kSumRegs; ++k) sum[k] = hand[k][lane];
+      finish_rows<kA, kPass, kN>(d, b, bin, lo, hi, sum, rbase, wc);
+      const float r = warp_sums(sum);
+      if (lane < kSums) row[lane] = r;
+    }
+    if (kPass == kPassSplit && lane == 0) sh.count[s][lw][part] = wc;
+  }
+}
+
+template <class T, int kA, int kPass>
+__device__ __noinline__ void team_item(const PairDesc* d, const LevelMaps& maps, int li, int vw, int lw,
+                                       int part, int chunk, const KParams& P, TeamShared& sh, int s,
+                                       unsigned* sh_hist, int lo, int hi, float* row) {
+  const LevelMaps L = maps;  // in registers: the caller's copy lies in its stack frame
+  static_assert(level_chunk(0) == 16 * kBlock && level_chunk(1) == 8 * kBlock && level_chunk(2) == 4 * kBlock &&
+                    level_chunk(3) == 4 * kBlock, "pixels of a lane per level");
+  if (chunk == 16 * kBlock)
+    team_batch<T, kA, kPass, 8>(d, L, li, vw, lw, part, chunk, P, sh, s, sh_hist, lo, hi, row);
+  else if (chunk == 8 * kBlock)
+    team_batch<T, kA, kPass, 4>(d, L, li, vw, lw, part, chunk, P, sh, s, sh_hist, lo, hi, row);
+  else
+    team_batch<T, kA, kPass, 2>(d, L, li, vw, lw, part, chunk, P, sh, s, sh_hist, lo, hi, row);
+}
+
+// The recorded rows of one item warp with klo <= bin <= khi, added in packed
+// order (fix_consume's): record i of the c0 + c1 lies in part 0's places up to
+// c0, then in part 1's. issue() sends for the first 64.
+struct TeamFix {
+  int c0, total, base, half;
+  float4 r0[kFixR], r1[kFixR];
+  __device__ __forceinline__ void issue(const PairDesc* d, int e0) {
+#pragma unroll
+    for (int r = 0; r < kFixR; ++r) {
+      const int i = e0 + r * 32 + (threadIdx.x & 31);
+      if (i < total) {
+        const size_t at = base + (i < c0 ? i : half + i - c0);
+        r0[r] = __ldcg(d->recs + 2 * at);
+        r1[r] = __ldcg(d->recs + 2 * at + 1);
+      }
+    }
+  }
+  __device__ __forceinline__ void begin(const PairDesc* d, int li, int vw, int chunk, const int (&count)[2]) {
+    c0 = count[0];
+    total = c0 + count[1];
+    base = li * chunk + vw * (chunk / kBlockWarps);
+    half = chunk / kBlockWarps / 2;
+    issue(d, 0);
+  }
+  __device__ __forceinline__ float finish(const PairDesc* d, int klo, int khi) {
+    float sum[kSumRegs];
+    zero_sums(sum);
+    for (int e0 = 0; e0 < total;) {
+#pragma unroll
+      for (int r = 0; r < kFixR; ++r) {
+        if (e0 + r * 32 + (int)(threadIdx.x & 31) >= total) continue;
+        const int k = __float_as_int(r1[r].w);
+        if (k >= klo && k <= khi) {
+          const float a[6] = {r0[r].x, r0[r].y, r0[r].z, r0[r].w, r1[r].x, r1[r].y};
+          accumulate(a, r1[r].z, sum);
+        }
+      }
+      e0 += 32 * kFixR;
+      issue(d, e0);
+    }
+    return warp_sums(sum);
+  }
 };
 
 // The band around a median and whether it lies in the window [w0, w1).
@@ -233,6 +301,7 @@ template <class T, int kA>
 __device__ void team_work(const PairDesc* d, const TeamPair& tp, int w, unsigned long long limit_ns,
                           const KParams& P, TeamShared& sh, unsigned* sh_hist) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lw = warp % kTeamWarps, part = warp / kTeamWarps;
   int level = P.levels - 1, w0 = -1, w1 = -1;
   for (unsigned it = 0;; ++it) {
     const LevelMaps L = d->lv[level];
@@ -243,25 +312,26 @@ __device__ void team_work(const PairDesc* d, const TeamPair& tp, int w, unsigned
       unsigned pixels = 0;
       int s = 0;
       for (int hid = w; hid < halves; hid += tp.workers, ++s) {
-        const int li = hid >> 1, vw = (hid & 1) + 2 * warp;
+        const int li = hid >> 1, vw = (hid & 1) + 2 * lw;
         // the half item's pixels: 32-pixel groups vw, vw + 8, ... of the item
         const int ip = min(fn - li * chunk, chunk), rest = ip % kBlock;
         if (warp == 0)
           for (int k = 0; k < kTeamWarps; ++k)
             pixels += ip / kBlock * 32 + min(32, max(0, rest - ((hid & 1) + 2 * k) * 32));
-        int count = 0;
         if (w0 >= 0)
-          team_item<T, kA, kPassSplit>(d, L, li, vw, chunk, sh.xf, P, sh_hist, w0, w1, sh.row_a[s][warp], &count);
+          team_item<T, kA, kPassSplit>(d, L, li, vw, lw, part, chunk, P, sh, s, sh_hist, w0, w1, sh.row_a[s][lw]);
         else
-          team_item<T, kA, kPassHist>(d, L, li, vw, chunk, sh.xf, P, sh_hist, 0, 0, nullptr, &count);
-        if (lane == 0) sh.count[s][warp] = count;
+          team_item<T, kA, kPassHist>(d, L, li, vw, lw, part, chunk, P, sh, s, sh_hist, 0, 0, nullptr);
       }
+      const int slots = s;
       __syncthreads();
       flush_hist(sh_hist, hist, P.bins, pixels, &sh.matched);
-      // the first half item's recorded rows, on their way while the histogram
-      // completes
-      FixLoad f;
-      if (w0 >= 0) fix_issue(d, w >> 1, chunk, (w & 1) + 2 * warp, f);
+      // the recorded rows of each part's first slot, on their way while the
+      // histogram completes (the parts take the slots in turn)
+      TeamFix f;
+      auto item_of = [&](int slot) { return (w + slot * tp.workers) >> 1; };
+      auto warp_of = [&](int slot) { return ((w + slot * tp.workers) & 1) + 2 * lw; };
+      if (w0 >= 0 && part < slots) f.begin(d, item_of(part), warp_of(part), chunk, sh.count[part][lw]);
       if (warp == 0) {
         int N, kmed;
         const bool ok = warp_median(hist, P.bins, (unsigned)fn, limit_ns, N, kmed);
@@ -274,30 +344,33 @@ __device__ void team_work(const PairDesc* d, const TeamPair& tp, int w, unsigned
       if (sh.abort) return;
       if (!sh.stop) {
         const int hit = sh.hit, klo = sh.klo, khi = sh.khi;
-        s = 0;
-        for (int hid = w; hid < halves; hid += tp.workers, ++s) {
-          const int li = hid >> 1, vw = (hid & 1) + 2 * warp;
-          float* row = sh.row[s & 1][warp];
+        // rows of two slots at a time: on a hit a slot for each part, else the
+        // parts together on one slot after the other
+        for (int s0 = 0; s0 < slots; s0 += 2) {
           if (hit) {
-            float sum[kSumRegs];
-            zero_sums(sum);
-            if (s > 0) fix_issue(d, li, chunk, vw, f);
-            f.total = sh.count[s][warp];
-            fix_consume(d, li, chunk, vw, klo, khi, f, sum);
-            const float r = warp_sums(sum);
-            if (lane < kSums) row[lane] = __fadd_rn(sh.row_a[s][warp][lane], r);
+            s = s0 + part;
+            if (s < slots) {
+              if (s0 > 0) f.begin(d, item_of(s), warp_of(s), chunk, sh.count[s][lw]);
+              const float r = f.finish(d, klo, khi);
+              if (lane < kSums) sh.row[part][lw][lane] = __fadd_rn(sh.row_a[s][lw][lane], r);
+            }
           } else {
-            int count;
-            team_item<T, kA, kPassBand>(d, L, li, vw, chunk, sh.xf, P, nullptr, klo, khi, row, &count);
-            if (lane < kSums) row[lane] = __fadd_rn(0.f, row[lane]);
+            for (s = s0; s < min(s0 + 2, slots); ++s) {
+              float* row = sh.row[s & 1][lw];
+              team_item<T, kA, kPassBand>(d, L, item_of(s), warp_of(s), lw, part, chunk, P, sh, s, nullptr, klo,
+                                          khi, row);
+              if (part == 1 && lane < kSums) row[lane] = __fadd_rn(0.f, row[lane]);
+            }
           }
           __syncthreads();
           // the item's pairwise halving, as far as these four warps go
-          if (warp == 0 && lane < kSums) {
-            float (*r)[32] = sh.row[s & 1];
+          s = s0 + part;
+          if (lw == 0 && s < slots && lane < kSums) {
+            float (*r)[32] = sh.row[part];
             const float v = __fadd_rn(__fadd_rn(r[0][lane], r[2][lane]), __fadd_rn(r[1][lane], r[3][lane]));
-            packet_store(d->team_rows + (size_t)hid * 32 + lane, __float_as_uint(v), tp.tag + it);
+            packet_store(d->team_rows + (size_t)(w + s * tp.workers) * 32 + lane, __float_as_uint(v), tp.tag + it);
           }
+          if (s0 + 2 < slots) __syncthreads();  // the rows are free again
         }
       }
     }
@@ -339,6 +412,11 @@ __device__ void team_lead(const PairDesc* d, const TeamPair& tp, const PairInput
     init_state(d, in, P, sT);
   }
   __syncthreads();
+  // what every solve takes, kept by warp 0
+  const SolveLane sl = solve_lane();
+  double Tmc[3], Tmt[3];
+  load_tm(d->Tm, Tmc, Tmt);
+  const double lam2c = 2.0 * in.lambda;
   int level = P.levels - 1, w0 = -1, w1 = -1;
   for (unsigned it = 0;; ++it) {
     const int chunk = level_chunk(level), fn = d->lv[level].fw * d->lv[level].fh;
@@ -367,6 +445,8 @@ __device__ void team_lead(const PairDesc* d, const TeamPair& tp, const PairInput
     __syncthreads();
     if (sh.abort) return;
     if (!sh.stop) {
+      NextStep next = {};
+      if (warp == 0) next = next_step(pre, level, P);
       // per sum (lane) the items' values: sub-sums over items sub, sub + 8, ...
       // (combine_and_solve's order)
       ItemSum (*part)[kSums] = reinterpret_cast<ItemSum (*)[kSums]>(sh.part);
@@ -374,10 +454,9 @@ __device__ void team_lead(const PairDesc* d, const TeamPair& tp, const PairInput
       const unsigned long long want = tp.tag + it;
       Wait wait;
       bool ok = true;
-      // a warp reads its two sub-sums' packets together: one round trip covers
-      // 80 items (a 640x480 frame has 75), where one after the other with eight
-      // items in flight took four
-      constexpr int kSubs = kBlockWarps / kTeamWarps, kFly = 10;
+      // a warp reads its sub-sum's packets together: one round trip covers 80
+      // items (a 640x480 frame has 75)
+      constexpr int kLeadWarps = kTeamBlock / 32, kSubs = kBlockWarps / kLeadWarps, kFly = 10;
       ItemSum sub[kSubs];
       for (int l0 = warp; l0 < count && ok; l0 += kFly * kBlockWarps) {
         unsigned long long a[kSubs][kFly], b[kSubs][kFly];
@@ -387,7 +466,7 @@ __device__ void team_lead(const PairDesc* d, const TeamPair& tp, const PairInput
           for (int j = 0; j < kSubs; ++j)
 #pragma unroll
             for (int i = 0; i < kFly; ++i) {
-              const int l = l0 + j * kTeamWarps + i * kBlockWarps;
+              const int l = l0 + j * kLeadWarps + i * kBlockWarps;
               a[j][i] = b[j][i] = want << 32;
               if (l < count && lane < kSums) {
                 a[j][i] = packet_load(d->team_rows + (size_t)(2 * l) * 32 + lane);
@@ -408,11 +487,11 @@ __device__ void team_lead(const PairDesc* d, const TeamPair& tp, const PairInput
         for (int j = 0; j < kSubs; ++j)
 #pragma unroll
           for (int i = 0; i < kFly; ++i)
-            if (l0 + j * kTeamWarps + i * kBlockWarps < count)
+            if (l0 + j * kLeadWarps + i * kBlockWarps < count)
               sub[j].add(__fadd_rn(__uint_as_float((unsigned)a[j][i]), __uint_as_float((unsigned)b[j][i])), shift);
       }
       if (lane < kSums)
-        for (int j = 0; j < kSubs; ++j) part[warp + j * kTeamWarps][lane] = sub[j];
+        for (int j = 0; j < kSubs; ++j) part[warp + j * kLeadWarps][lane] = sub[j];
       if (!ok) sh.abort = 1;
       __syncthreads();
       if (sh.abort) return;
@@ -433,8 +512,8 @@ __device__ void team_lead(const PairDesc* d, const TeamPair& tp, const PairInput
             sh.w1 = nw1;
           }
         };
-        const int next = solve_update(d, st, sh.sums, level, P, sh.hit ? 1 : 2, pre, Tc, publish);
-        if (__shfl_sync(0xffffffffu, next, 0) == -2) publish(Solved{}, -1, -1, -1);
+        if (solve_update(d, st, sh.sums, level, P, sh.hit ? 1 : 2, pre, next, sl, lam2c, Tc, Tmc, Tmt, publish) == -2)
+          publish(Solved{}, -1, -1, -1);
       } else {
         // every worker has read this histogram (its sums are here): empty it
         for (int b = threadIdx.x - 32; b < team_hist_words(P.bins); b += kTeamBlock - 32) hist[b] = 0u;
@@ -459,7 +538,7 @@ __device__ void team_lead(const PairDesc* d, const TeamPair& tp, const PairInput
 }
 
 template <class T, int kA>
-__global__ void __launch_bounds__(kTeamBlock, 2) k_icp_team(const __grid_constant__ TeamArgs A,
+__global__ void __launch_bounds__(kTeamBlock, 1) k_icp_team(const __grid_constant__ TeamArgs A,
                                                             const __grid_constant__ KParams P) {
   extern __shared__ unsigned sh_hist[];
   __shared__ __align__(16) TeamShared sh;
@@ -491,7 +570,9 @@ int team_blocks(const KParams& P) {
   int dev = 0, sms = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-#define KF_X(T, A) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_icp_team<T, A>, kTeamBlock, sm)
+#define KF_X(T, A)                                                                              \
+  cudaFuncSetAttribute(k_icp_team<T, A>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm); \
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_icp_team<T, A>, kTeamBlock, sm)
   KF_ASSOC_SWITCH(P, KF_X);
 #undef KF_X
   return sms * per;
