@@ -7,8 +7,10 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "kf_internal.cuh"
@@ -225,6 +227,34 @@ cudaError_t tmalloc(kf_tracker* t, T** p, size_t bytes) {
     *p = static_cast<T*>(q);
   }
   return e;
+}
+
+// Grid sizes of the tracker's launches: occupancy queries, asked once per device
+// and kernel variant (a batch creates its trackers one after the other).
+void launch_sizes(kf_tracker* t) {
+  struct Sizes {
+    int device, precision, angle, shoot, bins;
+    int assoc, reduce, sched, team;
+  };
+  static std::mutex mutex;
+  static std::vector<Sizes> known;
+  const KParams& P = t->kp;
+  icp_attributes(P);
+  std::lock_guard<std::mutex> lock(mutex);
+  auto it = std::find_if(known.begin(), known.end(), [&](const Sizes& s) {
+    return s.device == t->device && s.precision == P.precision && s.angle == P.use_angle &&
+           s.shoot == (P.shoot_w > 0) && s.bins == P.bins;
+  });
+  if (it == known.end()) {
+    Sizes s = {t->device, P.precision, P.use_angle, P.shoot_w > 0, P.bins, 0, 0, 0, 0};
+    icp_grids(P, &s.assoc, &s.reduce, &s.sched);
+    s.team = team_blocks(P);
+    it = known.insert(known.end(), s);
+  }
+  t->grid_assoc = it->assoc;
+  t->grid_reduce = it->reduce;
+  t->grid_sched = it->sched;
+  t->team_blocks = it->team;
 }
 
 bool intr_valid(const kf_intrinsics* K, int levels, int max_w, int max_h, std::string& why) {
@@ -641,50 +671,65 @@ kf_status kf_track_create(const kf_params* p, int max_w, int max_h, void* cuda_s
   const size_t px0 = (size_t)max_w * max_h;
   PairDesc& D = t->h_desc;
   D.levels = p->levels;
-  if ((e = tmalloc(t, &t->d_depth_raw, px0 * sizeof(float))) != cudaSuccess) return bail(e);
-  D.depth_raw = t->d_depth_raw;
-  for (int l = 0; l < p->levels; ++l) {
-    const size_t pl = (size_t)(max_w >> l) * (max_h >> l);
-    LevelMaps& L = D.lv[l];
-    if ((e = tmalloc(t, &L.fdepth, pl * sizeof(float))) != cudaSuccess) return bail(e);
-    if ((e = tmalloc(t, &L.fA, 4 * pl * t->elem)) != cudaSuccess) return bail(e);
-    if ((e = tmalloc(t, &L.fB, 2 * pl * t->elem)) != cudaSuccess) return bail(e);
-    if ((e = tmalloc(t, &L.mA, 4 * pl * t->elem)) != cudaSuccess) return bail(e);
-    if ((e = tmalloc(t, &L.mB, 2 * pl * t->elem)) != cudaSuccess) return bail(e);
-  }
-  t->max_items = (int)(((size_t)max_w * max_h + kChunk - 1) / kChunk);
-  if ((e = tmalloc(t, &t->d_state, sizeof(PairState))) != cudaSuccess) return bail(e);
-  if ((e = tmalloc(t, &D.hist, sizeof(unsigned) * p->hist_bins)) != cudaSuccess) return bail(e);
-  if ((e = tmalloc(t, &D.partials, sizeof(float) * kPartialStride * t->max_items)) != cudaSuccess) return bail(e);
+  t->max_items = (int)((px0 + kChunk - 1) / kChunk);
   D.partial_cap = t->max_items;
   D.px_cap = (int)px0;
-  if ((e = tmalloc(t, &D.counters, sizeof(unsigned) * 2)) != cudaSuccess) return bail(e);
-  if ((e = tmalloc(t, &D.recs, 2 * sizeof(float4) * (px0 + kChunk))) != cudaSuccess) return bail(e);
-  if ((e = tmalloc(t, &D.wcount, sizeof(unsigned) * kBlockWarps * t->max_items)) != cudaSuccess)
-    return bail(e);
-  if (t->max_items <= kTeamMaxItems) {
-    const size_t hist = sizeof(unsigned) * 3 * team_hist_words(p->hist_bins);
-    const size_t msg = (hist + 255) / 256 * 256, rows = msg + 32 * sizeof(unsigned long long);
-    t->team_bytes = rows + (size_t)t->max_items * 2 * 32 * sizeof(unsigned long long);
-    char* area = nullptr;
-    if ((e = tmalloc(t, &area, t->team_bytes)) != cudaSuccess) return bail(e);
-    if ((e = cudaMemsetAsync(area, 0, t->team_bytes, t->stream)) != cudaSuccess) return bail(e);
-    t->d_team = area;
-    D.team_hist = reinterpret_cast<unsigned*>(area);
-    D.team_msg = reinterpret_cast<unsigned long long*>(area + msg);
-    D.team_rows = reinterpret_cast<unsigned long long*>(area + rows);
-    t->team_blocks = team_blocks(t->kp);
-  }
-  if ((e = tmalloc(t, &t->d_desc, sizeof(PairDesc))) != cudaSuccess) return bail(e);
-  if ((e = tmalloc(t, &t->d_self, sizeof(PairDesc*))) != cudaSuccess) return bail(e);
-  if ((e = tmalloc(t, &t->d_dbg_list, sizeof(int) * list_ints(1))) != cudaSuccess) return bail(e);
-  if ((e = tmalloc(t, &t->d_dbg_counter, sizeof(unsigned))) != cudaSuccess) return bail(e);
-  if ((e = cudaMemsetAsync(t->d_dbg_counter, 0, sizeof(unsigned), t->stream)) != cudaSuccess) return bail(e);
-  icp_grids(t->kp, &t->grid_assoc, &t->grid_reduce, &t->grid_sched);
-  if ((e = tmalloc(t, &t->d_dbg_pose, sizeof(double) * 16)) != cudaSuccess) return bail(e);
+  // two allocations, cut into 256-byte aligned parts: what starts at zero, and
+  // the maps (an allocation each made creation mostly allocation calls)
+  const bool team = t->max_items <= kTeamMaxItems;
+  char* base = nullptr;
+  size_t at = 0;
+  auto part = [&](auto** ptr, size_t bytes) {
+    *ptr = base ? reinterpret_cast<std::remove_reference_t<decltype(*ptr)>>(base + at) : nullptr;
+    at += (bytes + 255) / 256 * 256;
+  };
+  auto zeroed = [&] {
+    at = 0;
+    part(&t->d_state, sizeof(PairState));
+    part(&D.counters, sizeof(unsigned) * 2);
+    part(&t->d_dbg_counter, sizeof(unsigned));
+    part(&D.hist, sizeof(unsigned) * p->hist_bins);
+    part(&t->d_desc, sizeof(PairDesc));
+    part(&t->d_self, sizeof(PairDesc*));
+    part(&t->d_dbg_list, sizeof(int) * list_ints(1));
+    part(&t->d_dbg_pose, sizeof(double) * 16);
+    if (team) {
+      const size_t first = at;
+      part(&D.team_hist, sizeof(unsigned) * 3 * team_hist_words(p->hist_bins));
+      part(&D.team_msg, 32 * sizeof(unsigned long long));
+      part(&D.team_rows, (size_t)t->max_items * 2 * 32 * sizeof(unsigned long long));
+      t->d_team = D.team_hist;
+      t->team_bytes = at - first;
+    }
+  };
+  auto maps = [&] {
+    at = 0;
+    part(&t->d_depth_raw, px0 * sizeof(float));
+    for (int l = 0; l < p->levels; ++l) {
+      const size_t pl = (size_t)(max_w >> l) * (max_h >> l);
+      LevelMaps& L = D.lv[l];
+      part(&L.fdepth, pl * sizeof(float));
+      part(reinterpret_cast<char**>(&L.fA), 4 * pl * t->elem);
+      part(reinterpret_cast<char**>(&L.fB), 2 * pl * t->elem);
+      part(reinterpret_cast<char**>(&L.mA), 4 * pl * t->elem);
+      part(reinterpret_cast<char**>(&L.mB), 2 * pl * t->elem);
+    }
+    part(&D.partials, sizeof(float) * kPartialStride * t->max_items);
+    part(&D.wcount, sizeof(unsigned) * kBlockWarps * t->max_items);
+    part(&D.recs, 2 * sizeof(float4) * (px0 + kChunk));
+  };
+  maps();  // sizes first, then the parts' addresses
+  if ((e = tmalloc(t, &base, at)) != cudaSuccess) return bail(e);
+  maps();
+  base = nullptr;
+  zeroed();
+  const size_t zero_bytes = at;
+  if ((e = tmalloc(t, &base, zero_bytes)) != cudaSuccess) return bail(e);
+  zeroed();
+  if ((e = cudaMemsetAsync(base, 0, zero_bytes, t->stream)) != cudaSuccess) return bail(e);
+  D.depth_raw = t->d_depth_raw;
+  launch_sizes(t);
   D.st = t->d_state;
-  if ((e = cudaMemsetAsync(t->d_state, 0, sizeof(PairState), t->stream)) != cudaSuccess) return bail(e);
-  if ((e = cudaMemsetAsync(D.counters, 0, sizeof(unsigned) * 2, t->stream)) != cudaSuccess) return bail(e);
   if ((e = cudaMemcpyAsync(t->d_desc, &D, sizeof(PairDesc), cudaMemcpyHostToDevice, t->stream)) != cudaSuccess) return bail(e);
   const PairDesc* self = t->d_desc;
   if ((e = cudaMemcpyAsync(t->d_self, &self, sizeof(self), cudaMemcpyHostToDevice, t->stream)) != cudaSuccess) return bail(e);
@@ -866,7 +911,6 @@ kf_status kf_set_model(kf_tracker* t, const float* vertex, const float* normal,
       for (int j = 0; j < 4; ++j) t->h_desc.Tm[i * 4 + j] = model_pose[i * 4 + j];
     double fx = K->fx, fy = K->fy, cx = K->cx, cy = K->cy;
     int w = K->width, h = K->height;
-    int mw[KF_MAX_LEVELS], mh[KF_MAX_LEVELS];
     for (int l = 0; l < t->p.levels; ++l) {
       if (l > 0) {  // model level l+1 = level l at even pixels: f / 2, c / 2
         w /= 2;
@@ -877,17 +921,14 @@ kf_status kf_set_model(kf_tracker* t, const float* vertex, const float* normal,
         cy /= 2;
       }
       LevelMaps& L = t->h_desc.lv[l];
-      L.mw = mw[l] = w;
-      L.mh = mh[l] = h;
+      L.mw = w;
+      L.mh = h;
       L.mfx = (float)fx;
       L.mfy = (float)fy;
       L.mcx = (float)cx;
       L.mcy = (float)cy;
     }
-    kf_status st = upload_desc(t, s);
-    if (st != KF_OK) return st;
-    KF_CK(t, launch_model_prep(t->d_desc, V, N, K->width, K->height, t->p.levels, mw, mh,
-                               t->p.precision, nullptr, s));
+    KF_CK(t, launch_model_prep(t->h_desc, t->d_desc, V, N, K->width, K->height, t->p.precision, s));
     if (!is_device_ptr) KF_CK(t, cudaStreamSynchronize(s));
     t->has_model = true;
     return KF_OK;

@@ -20,23 +20,41 @@ constexpr int kTx = 32, kTy = 8;
 
 __device__ __forceinline__ bool valid_depth(float z) { return isfinite(z) && z > 0.f; }
 
-// Model level l = level-0 model maps at pixels (x 2^l, y 2^l), as records; a pixel is a hole (NaN vertex and normal) when any component is
-// non-finite or the normal is all zero.
+// Model level l = level-0 model maps at pixels (x 2^l, y 2^l), as records; a
+// pixel is a hole (NaN vertex and normal) when any component is non-finite or
+// the normal is all zero. One launch, each pixel read once and written to every
+// level it belongs to; it also brings the pair's descriptor on the device up
+// to date (its copy `desc` comes with the launch), which a copy of its own would
+// take longer to queue than this kernel runs.
 template <class T>
-__global__ void __launch_bounds__(kTx* kTy) k_model_prep(const PairDesc* d, const float* Vin,
-                                                         const float* Nin, int w, int level) {
-  const LevelMaps& L = d->lv[level];
+__global__ void __launch_bounds__(kTx* kTy) k_model_prep(const __grid_constant__ PairDesc desc, PairDesc* d_desc,
+                                                         const float* Vin, const float* Nin, int w, int h) {
+  const int tid = threadIdx.y * kTx + threadIdx.x;
+  if (blockIdx.x == 0 && blockIdx.y == 0) {
+    constexpr int kWords = sizeof(PairDesc) / sizeof(unsigned long long);
+    static_assert(sizeof(PairDesc) % sizeof(unsigned long long) == 0 && kWords <= kTx * kTy, "descriptor size");
+    if (tid < kWords)
+      reinterpret_cast<unsigned long long*>(d_desc)[tid] = reinterpret_cast<const unsigned long long*>(&desc)[tid];
+  }
   const int x = blockIdx.x * kTx + threadIdx.x, y = blockIdx.y * kTy + threadIdx.y;
-  if (x >= L.mw || y >= L.mh) return;
-  const long src = ((long)(y << level) * w + (x << level)) * 3;
-  const float vx = Vin[src], vy = Vin[src + 1], vz = Vin[src + 2];
-  const float nx = Nin[src], ny = Nin[src + 1], nz = Nin[src + 2];
+  if (x >= w || y >= h) return;
+  const long src = ((long)y * w + x) * 3;
+  const float vx = __ldg(Vin + src), vy = __ldg(Vin + src + 1), vz = __ldg(Vin + src + 2);
+  const float nx = __ldg(Nin + src), ny = __ldg(Nin + src + 1), nz = __ldg(Nin + src + 2);
   const bool ok = isfinite(vx) && isfinite(vy) && isfinite(vz) && isfinite(nx) && isfinite(ny) &&
                   isfinite(nz) && (nx != 0.f || ny != 0.f || nz != 0.f);
   const float nan = __int_as_float(0x7fc00000);
-  const int i = y * L.mw + x;
-  Store<T>::store_a(L.mA, i, ok ? make_float4(vx, vy, vz, nx) : make_float4(nan, nan, nan, nan));
-  Store<T>::store_b(L.mB, i, ok ? make_float2(ny, nz) : make_float2(nan, nan));
+  const float4 a = ok ? make_float4(vx, vy, vz, nx) : make_float4(nan, nan, nan, nan);
+  const float2 b = ok ? make_float2(ny, nz) : make_float2(nan, nan);
+#pragma unroll
+  for (int l = 0; l < KF_MAX_LEVELS; ++l) {
+    if (l >= desc.levels || ((x | y) & ((1 << l) - 1)) != 0) break;
+    const LevelMaps& L = desc.lv[l];
+    const int xl = x >> l, yl = y >> l;
+    if (xl >= L.mw || yl >= L.mh) break;
+    Store<T>::store_a(L.mA, yl * L.mw + xl, a);
+    Store<T>::store_b(L.mB, yl * L.mw + xl, b);
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -312,7 +330,6 @@ __global__ void __launch_bounds__(kTx* kTy, KF_FE_MINB) k_frontend_fused(DescLis
   if (levels > 3) write_maps<T, kTile / 8, 1>(d->lv[3], s_d3, R0 >> 3, X0 >> 3, Y0 >> 3);
 }
 
-dim3 grid_for(int w, int h, int n) { return dim3((w + kTx - 1) / kTx, (h + kTy - 1) / kTy, n); }
 
 // ---------------------------------------------------------------------------
 // Integral-image normals (Sec. 3.3; Holzer et al.): the average 3D gradient
@@ -612,17 +629,11 @@ cudaError_t launch_integral_normals(const DescList& list, int max_w, int max_h, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_model_prep(const PairDesc* d_desc, const float* V, const float* N, int w,
-                              int h, int levels, const int* mw, const int* mh, int precision,
-                              const LevelMaps* /*host_levels*/, cudaStream_t s) {
-  (void)h;
-  const dim3 blk(kTx, kTy);
-  for (int l = 0; l < levels; ++l) {
-    if (precision == KF_FP16)
-      k_model_prep<__half><<<grid_for(mw[l], mh[l], 1), blk, 0, s>>>(d_desc, V, N, w, l);
-    else
-      k_model_prep<float><<<grid_for(mw[l], mh[l], 1), blk, 0, s>>>(d_desc, V, N, w, l);
-  }
+cudaError_t launch_model_prep(const PairDesc& desc, PairDesc* d_desc, const float* V, const float* N, int w,
+                              int h, int precision, cudaStream_t s) {
+  const dim3 blk(kTx, kTy), grid((w + kTx - 1) / kTx, (h + kTy - 1) / kTy);
+  if (precision == KF_FP16) k_model_prep<__half><<<grid, blk, 0, s>>>(desc, d_desc, V, N, w, h);
+  else k_model_prep<float><<<grid, blk, 0, s>>>(desc, d_desc, V, N, w, h);
   return cudaGetLastError();
 }
 

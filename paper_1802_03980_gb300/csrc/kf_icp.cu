@@ -1069,12 +1069,21 @@ int wave(K kernel, size_t smem) {
   int dev = 0, sms = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, kBlock, smem);
   return sms * (per > 0 ? per : 1);
 }
 
 }  // namespace
+
+void icp_attributes(const KParams& P) {
+  const int sm = P.bins * (int)sizeof(unsigned);
+#define KF_X(T, A)                                                                               \
+  cudaFuncSetAttribute(k_assoc_hist<T, A>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm); \
+  cudaFuncSetAttribute(k_icp_sched<T, A>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sched_smem<T, A>(P))
+  KF_ASSOC_SWITCH(P, KF_X);
+#undef KF_X
+  team_attributes(P);
+}
 
 void icp_grids(const KParams& P, int* g_assoc, int* g_reduce, int* g_sched) {
   const size_t sm = (size_t)P.bins * sizeof(unsigned);

@@ -311,9 +311,13 @@ cudaError_t launch_frontend(const DescList& list, int max_w, int max_h, int leve
 // front end): replaces the frame normals and drops vertices without one
 cudaError_t launch_integral_normals(const DescList& list, int max_w, int max_h, int levels,
                                     const KParams& P, cudaStream_t s);
-cudaError_t launch_model_prep(const PairDesc* d_desc, const float* V, const float* N, int w,
-                              int h, int levels, const int* mw, const int* mh, int precision,
-                              const LevelMaps* host_levels, cudaStream_t s);
+// the model's records of every level, and the pair's device descriptor := desc
+cudaError_t launch_model_prep(const PairDesc& desc, PairDesc* d_desc, const float* V, const float* N, int w,
+                              int h, int precision, cudaStream_t s);
+// the shared memory that the variant's kernels may take (before any query or
+// launch of them in a context)
+void icp_attributes(const KParams& P);
+void team_attributes(const KParams& P);
 // grid sizes (one wave) of the per-stage and the scheduled ICP kernels
 void icp_grids(const KParams& P, int* g_assoc, int* g_reduce, int* g_sched);
 cudaError_t launch_icp_init(const PairDesc* const* descs, const PairInput* in, int n, int* list,

@@ -565,14 +565,20 @@ __global__ void __launch_bounds__(kTeamBlock, 1) k_icp_team(const __grid_constan
 
 }  // namespace
 
+void team_attributes(const KParams& P) {
+#define KF_X(T, A)                                                                     \
+  cudaFuncSetAttribute(k_icp_team<T, A>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                       P.bins * (int)sizeof(unsigned))
+  KF_ASSOC_SWITCH(P, KF_X);
+#undef KF_X
+}
+
 int team_blocks(const KParams& P) {
   const int sm = P.bins * (int)sizeof(unsigned);
   int dev = 0, sms = 0, per = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-#define KF_X(T, A)                                                                              \
-  cudaFuncSetAttribute(k_icp_team<T, A>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm); \
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_icp_team<T, A>, kTeamBlock, sm)
+#define KF_X(T, A) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_icp_team<T, A>, kTeamBlock, sm)
   KF_ASSOC_SWITCH(P, KF_X);
 #undef KF_X
   return sms * per;
