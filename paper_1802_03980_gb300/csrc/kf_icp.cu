@@ -277,7 +277,7 @@ __device__ void assoc_items(const PairDesc* d, const LevelMaps& L, int first, in
 // (cp.async.wait_group): no barrier. The same pixels in the same order as
 // assoc_items: the same sums.
 // Measured on GB300, the whole alignment of a batch, register gathers -> ring:
-// 256 pairs 640x480 3.92 -> 3.55 ms, 64 mixed pairs float16 2.27 -> 2.03 ms, 32
+// 256 pairs 640x480 3.92 -> 3.55 ms (3.31 since), 64 mixed pairs float16 2.27 -> 2.03 ms, 32
 // pairs 0.85 -> 0.81 ms. Two pixels a batch: one pixel 4.2 ms (256 pairs), four
 // 3.74 (its registers); model records two or three batches ahead 3.53, 3.57; 24
 // warps on an SM 5.3 (spills).
@@ -378,6 +378,10 @@ __device__ void assoc_ring(const PairDesc* d, const LevelMaps& L, int first, int
   float sum[kSumRegs];
   zero_sums(sum);
   int wc = 0, fs = 0, ms = 0;  // the ring places of the batch being summed
+  // the item of the batch, where it ends and the warp's record region in it,
+  // stepped: dividing by the item's size twice a batch cost 7 % (256 pairs
+  // 640x480 3.55 ms, now 3.31)
+  int li = first, ie = begin + chunk, rbase = begin + warp * (chunk / kBlockWarps);
   for (int b0 = begin; b0 < end; b0 += kPixels) {
     // the batch kAhead later: its frame records have come (one model group
     // stands behind them); the frame records after them take the free place
@@ -414,11 +418,9 @@ __device__ void assoc_ring(const PairDesc* d, const LevelMaps& L, int first, int
       for (int u = 0; u < kN; ++u) j[k][u] = j[k + 1][u];
     fs = fs + 1 < kAhead + 2 ? fs + 1 : 0;
     ms = ms < kAhead ? ms + 1 : 0;
-    const int li = b0 / chunk;
-    const int rbase = li * chunk + warp * (chunk / kBlockWarps);
     finish_batch<0, kPass, 0>(d, b0, end, t, cur, sxf, P, sh_hist, lo, hi, sum, rbase, wc);
     const int after = b0 + kPixels;
-    if (after >= end || after % chunk == 0) {  // the item's last batch
+    if (after >= end || after == ie) {  // the item's last batch
       if constexpr (kPass == kPassSplit) {
         if ((t & 31) == 0) {
           KF_GUARD(li < d->partial_cap, 7, li, d->partial_cap)
@@ -431,6 +433,9 @@ __device__ void assoc_ring(const PairDesc* d, const LevelMaps& L, int first, int
         write_row(d, li, kPass == kPassBand, sum);
         zero_sums(sum);
       }
+      ++li;
+      ie += chunk;
+      rbase += chunk;
     }
   }
   copy_wait<0>();
