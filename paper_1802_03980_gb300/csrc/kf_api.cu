@@ -298,6 +298,8 @@ bool set_frame_levels(kf_tracker* t, const kf_intrinsics* K) {
     L.fh = h;
     L.ffx = (float)fx;
     L.ffy = (float)fy;
+    L.fifx = 1.f / L.ffx;
+    L.fify = 1.f / L.ffy;
     L.fcx = (float)cx;
     L.fcy = (float)cy;
   }

@@ -75,11 +75,15 @@ __global__ void __launch_bounds__(kTx* kTy) k_model_prep(const __grid_constant__
 //    whether a frame pixel takes part.
 // ---------------------------------------------------------------------------
 constexpr int kTile = 32;
-constexpr int kRMax = 40 + 2 * 4;  // largest raw region: 4 levels, bilateral radius 4
 
-__device__ __forceinline__ int region0(int levels) {
-  return ((kTile >> (levels - 1)) + 1) << (levels - 1);
-}
+// side of the level-0 region that is filtered, and of the raw region around it
+__host__ __device__ constexpr int region0(int levels) { return ((kTile >> (levels - 1)) + 1) << (levels - 1); }
+
+// Row stride of the raw region's pairs, from its side RR on: half the filtered
+// region's side R0 modulo 8, so that a warp whose 32 pixels go on in the
+// region's next row of pairs reads the other banks there (without it a third of
+// the filter's shared-memory wavefronts were conflicts).
+__host__ __device__ constexpr int pair_stride(int R0, int RR) { return RR + (((R0 + 1) / 2 - RR) % 8 + 8) % 8; }
 
 // Calls f(lx, ly) for the cells t = tid, tid + nthr, ... of a w x h region
 // in row-major order, stepping the coordinates instead of dividing t.
@@ -87,6 +91,7 @@ template <class F>
 __device__ __forceinline__ void for_region(int w, int h, int tid, int nthr, F f) {
   const int q = nthr / w, r = nthr - q * w;
   int ly = tid / w, lx = tid - ly * w;
+#pragma unroll 1
   while (ly < h) {
     f(lx, ly);
     lx += r;
@@ -109,17 +114,18 @@ __device__ __forceinline__ bool back_project(float ux, float uy, float ifx, floa
 
 // Maps of a level's tile x tile pixels from (ox, oy) on. A thread takes kRows
 // pixels below one another: the column's coordinates are formed once, and a
-// pixel's lower neighbour is the next pixel. Ds: level depth region of R x R
+// pixel's lower neighbour is the next pixel. The block's threads from kFirst on
+// take part. Ds: level depth region of R x R
 // whose origin is level pixel (ox, oy).
-template <class T, int kTileL, int kRows>
+template <class T, int kTileL, int kRows, int kFirst = 0>
 __device__ __forceinline__ void write_maps(const LevelMaps& Lg, const float* Ds, int R, int ox, int oy) {
   // a local copy: the map stores below could alias the descriptor in global
   // memory, which would force its fields to be reloaded for every pixel
   const LevelMaps L = Lg;
   const float nan = __int_as_float(0x7fc00000);
-  const float ifx = __fdiv_rn(1.f, L.ffx), ify = __fdiv_rn(1.f, L.ffy);
-  const int tid = threadIdx.y * kTx + threadIdx.x;
-  if (tid >= kTileL * kTileL / kRows) return;
+  const float ifx = L.fifx, ify = L.fify;
+  const int tid = threadIdx.y * kTx + threadIdx.x - kFirst;
+  if (tid < 0 || tid >= kTileL * kTileL / kRows) return;
   const int lx = tid % kTileL, ly0 = tid / kTileL * kRows;
   const int x = ox + lx;
   if (x >= L.fw) return;
@@ -223,45 +229,72 @@ __device__ __forceinline__ float bilateral_at(const float* s_raw, int RR, int cx
   return __fdividef(num, den);
 }
 
-template <class T, int RB>  // RB: the bilateral radius (a template so each launch holds one window)
+// RB: the bilateral radius. kLv: the number of levels, or 0 for any (read from
+// the descriptor). What bounds a batch is instruction issue (78 % of the slots,
+// 476 instructions a level-0 pixel before the levels were known here, a third of
+// them integer and compare): with the regions' sizes as constants their
+// divisions, 45 instructions a thread and phase, go; so do the halves of 1 / f
+// and of the pyramid's means, and a bounds check and two stores a raw pixel.
+// Measured on GB300, 256 frames 640x480, three levels: 1217 -> 867 us.
+template <class T, int RB, int kLv>
 __global__ void __launch_bounds__(kTx* kTy, KF_FE_MINB) k_frontend_fused(DescList list, KParams P) {
-#if KF_FE_PAIRS
-  // raw depth as vertical pairs: s_pair[y RR + x] = (D(x, y), D(x, y + 1)),
+  constexpr int r = RB;                                          // = P.bil_radius
+  constexpr int kR0 = region0(kLv > 0 ? kLv : KF_MAX_LEVELS);    // largest of the instance
+  constexpr int kRR = kR0 + 2 * r;
+  constexpr int nthr = kTx * kTy;
+  // raw depth as vertical pairs: s_pair[y S + x] = (D(x, y), D(x, y + 1)),
   // the row below the region holding no depth
-  __shared__ float2 s_pair[kRMax * kRMax];
+  constexpr int kStride = kLv > 0 ? pair_stride(kR0, kRR) : kRR + 7;  // the largest of the instance
+#if KF_FE_PAIRS
+  __shared__ float2 s_pair[kRR * kStride];
 #else
-  __shared__ float s_raw[kRMax * kRMax];
+  __shared__ float s_raw[kRR * kStride];
 #endif
-  __shared__ float s_d0[40 * 40];
-  __shared__ float s_d1[20 * 20];
-  __shared__ float s_d2[10 * 10];
-  __shared__ float s_d3[5 * 5];
+  __shared__ __align__(8) float s_d0[kR0 * kR0];
+  __shared__ __align__(8) float s_d1[kR0 / 2 * (kR0 / 2)];
+  __shared__ __align__(8) float s_d2[kR0 / 4 * (kR0 / 4)];
+  __shared__ __align__(8) float s_d3[kR0 / 8 * (kR0 / 8)];
   const PairDesc* d = list.d[blockIdx.z];
   const int W = d->iw, H = d->ih;
   const int X0 = blockIdx.x * kTile, Y0 = blockIdx.y * kTile;
   if (X0 >= W || Y0 >= H) return;
-  const int levels = d->levels;
-  const int R0 = region0(levels);
-  constexpr int r = RB;  // = P.bil_radius (the launch picks the instance)
+  const int levels = kLv > 0 ? kLv : d->levels;
+  const int R0 = kLv > 0 ? kR0 : region0(levels);
   const int RR = R0 + 2 * r;
-  const int nthr = blockDim.x * blockDim.y;
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+  const int S = pair_stride(R0, RR);
+  const int tid = threadIdx.y * kTx + threadIdx.x;
   const float* D = list.depth[blockIdx.z];
-  for_region(RR, RR, tid, nthr, [&](int lx, int ly) {
-    const int x = X0 - r + lx, y = Y0 - r + ly;
-    float z = kNoDepth;
-    if (x >= 0 && x < W && y >= 0 && y < H) {
-      z = __ldg(D + y * W + x);
-      if (!valid_depth(z)) z = kNoDepth;
+  // a thread loads a piece of a column, all of it before the first use: a pixel
+  // is the lower half of its own pair and the upper half of the one above
+  {
+    const int groups = nthr / RR, rows = (RR + groups - 1) / groups;
+    constexpr int kRows = (kRR + nthr / kRR - 1) / (nthr / kRR);  // the largest rows of the instance
+    const int lx = tid % RR, y0 = tid / RR * rows;
+    const int x = X0 - r + lx;
+    const bool xin = tid < groups * RR && (unsigned)x < (unsigned)W;
+    const int i0 = (Y0 - r + y0) * W + x;
+    float z[kRows + 1];
+#pragma unroll
+    for (int k = 0; k <= kRows; ++k) {
+      const int ly = y0 + k, y = Y0 - r + ly;
+      z[k] = kNoDepth;
+      if (xin && k <= rows && ly < RR && (unsigned)y < (unsigned)H) z[k] = __ldg(D + i0 + k * W);
     }
+#pragma unroll
+    for (int k = 0; k <= kRows; ++k)
+      if (!valid_depth(z[k])) z[k] = kNoDepth;
+    if (tid < groups * RR) {
+#pragma unroll
+      for (int k = 0; k < kRows; ++k)
+        if (k < rows && y0 + k < RR) {
 #if KF_FE_PAIRS
-    s_pair[ly * RR + lx].x = z;
-    if (ly > 0) s_pair[(ly - 1) * RR + lx].y = z;
-    if (ly == RR - 1) s_pair[ly * RR + lx].y = kNoDepth;
+          s_pair[(y0 + k) * S + lx] = make_float2(z[k], z[k + 1]);
 #else
-    s_raw[ly * RR + lx] = z;
+          s_raw[(y0 + k) * S + lx] = z[k];
 #endif
-  });
+        }
+    }
+  }
   __syncthreads();
   // bilateral filter over the R0 x R0 region: w = 2^(sw2 - dz^2 c2), the
   // k_bilateral weight with the exponent pre-scaled by log2(e)
@@ -271,8 +304,8 @@ __global__ void __launch_bounds__(kTx* kTy, KF_FE_MINB) k_frontend_fused(DescLis
   for_region(R0, (R0 + 1) >> 1, tid, nthr, [&](int lx, int py) {
     const int ly = 2 * py;
     const int x = X0 + lx, y = Y0 + ly;
-    const float2 z = s_pair[(ly + r) * RR + lx + r];
-    float2 out = RB > 0 ? bilateral_pair<RB>(s_pair, RR, lx + r, ly + r, z, P) : z;
+    const float2 z = s_pair[(ly + r) * S + lx + r];
+    float2 out = RB > 0 ? bilateral_pair<RB>(s_pair, S, lx + r, ly + r, z, P) : z;
     const bool xin = x < W;
     s_d0[ly * R0 + lx] = xin && y < H && z.x != kNoDepth ? out.x : 0.f;
     if (ly + 1 < R0) s_d0[(ly + 1) * R0 + lx] = xin && y + 1 < H && z.y != kNoDepth ? out.y : 0.f;
@@ -280,10 +313,10 @@ __global__ void __launch_bounds__(kTx* kTy, KF_FE_MINB) k_frontend_fused(DescLis
 #else
   for_region(R0, R0, tid, nthr, [&](int lx, int ly) {
     const int x = X0 + lx, y = Y0 + ly;
-    const float z = s_raw[(ly + r) * RR + lx + r];
+    const float z = s_raw[(ly + r) * S + lx + r];
     float out = 0.f;
     if (x < W && y < H && z != kNoDepth) {
-      out = RB > 0 ? bilateral_at<RB>(s_raw, RR, lx + r, ly + r, z, P) : z;
+      out = RB > 0 ? bilateral_at<RB>(s_raw, S, lx + r, ly + r, z, P) : z;
     }
     s_d0[ly * R0 + lx] = out;
   });
@@ -291,43 +324,43 @@ __global__ void __launch_bounds__(kTx* kTy, KF_FE_MINB) k_frontend_fused(DescLis
   __syncthreads();
   // pyramid: level l+1 from level l inside shared memory (same rule as k_downsample)
   float* lev[4] = {s_d0, s_d1, s_d2, s_d3};
-  for (int l = 0; l + 1 < levels; ++l) {
-    const int Rs = R0 >> l, Ro = R0 >> (l + 1);
+#pragma unroll
+  for (int l = 0; l + 1 < KF_MAX_LEVELS; ++l) {
+    if (l + 1 >= levels) break;
+    const int Rs = R0 >> l, Ro = R0 >> (l + 1);  // Rs is even
     const LevelMaps& Lo = d->lv[l + 1];
+    const int fw = Lo.fw, fh = Lo.fh;
     const int ox = X0 >> (l + 1), oy = Y0 >> (l + 1);
     const float* src = lev[l];
     float* dst = lev[l + 1];
     for_region(Ro, Ro, tid, nthr, [&](int lx, int ly) {
       float out = 0.f;
-      if (ox + lx < Lo.fw && oy + ly < Lo.fh) {
-        const float b[4] = {src[(2 * ly) * Rs + 2 * lx], src[(2 * ly) * Rs + 2 * lx + 1],
-                            src[(2 * ly + 1) * Rs + 2 * lx], src[(2 * ly + 1) * Rs + 2 * lx + 1]};
-        float anchor = 0.f;
-        bool have = false;
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-          if (!have && b[i] > 0.f) {
-            anchor = b[i];
-            have = true;
-          }
+      if (ox + lx < fw && oy + ly < fh) {
+        const float2 b0 = *reinterpret_cast<const float2*>(src + 2 * ly * Rs + 2 * lx);
+        const float2 b1 = *reinterpret_cast<const float2*>(src + (2 * ly + 1) * Rs + 2 * lx);
+        const float b[4] = {b0.x, b0.y, b1.x, b1.y};
+        // the first valid depth; none: no b[i] is counted
+        const float anchor = b[0] > 0.f ? b[0] : b[1] > 0.f ? b[1] : b[2] > 0.f ? b[2] : b[3];
         float s = 0.f;
         int c = 0;
 #pragma unroll
         for (int i = 0; i < 4; ++i)
-          if (have && b[i] > 0.f && fabsf(__fsub_rn(b[i], anchor)) <= P.thr3sr32) {
+          if (b[i] > 0.f && fabsf(__fsub_rn(b[i], anchor)) <= P.thr3sr32) {
             s = __fadd_rn(s, b[i]);
             ++c;
           }
-        out = c ? __fdiv_rn(s, (float)c) : 0.f;
+        // s / c: the products by 1/4, 1/2 and 1 round as the quotients do
+        out = c == 3 ? __fdiv_rn(s, 3.f) : __fmul_rn(s, c == 4 ? 0.25f : c == 2 ? 0.5f : 1.f);
       }
       dst[ly * Ro + lx] = out;
     });
     __syncthreads();
   }
+  // the coarser levels' pixels on different warps
   write_maps<T, kTile, 4>(d->lv[0], s_d0, R0, X0, Y0);
-  if (levels > 1) write_maps<T, kTile / 2, 1>(d->lv[1], s_d1, R0 >> 1, X0 >> 1, Y0 >> 1);
-  if (levels > 2) write_maps<T, kTile / 4, 1>(d->lv[2], s_d2, R0 >> 2, X0 >> 2, Y0 >> 2);
-  if (levels > 3) write_maps<T, kTile / 8, 1>(d->lv[3], s_d3, R0 >> 3, X0 >> 3, Y0 >> 3);
+  if (levels > 1) write_maps<T, kTile / 2, 2>(d->lv[1], s_d1, R0 >> 1, X0 >> 1, Y0 >> 1);
+  if (levels > 2) write_maps<T, kTile / 4, 1, 128>(d->lv[2], s_d2, R0 >> 2, X0 >> 2, Y0 >> 2);
+  if (levels > 3) write_maps<T, kTile / 8, 1, 192>(d->lv[3], s_d3, R0 >> 3, X0 >> 3, Y0 >> 3);
 }
 
 
@@ -416,7 +449,7 @@ __global__ void __launch_bounds__(kTx * kTy) k_ii_normals(DescList list, IiGrid 
   const int tid = threadIdx.y * kTx + threadIdx.x, nt = kTx * kTy;
   const int lane = threadIdx.x, warp = threadIdx.y;
   const float nan = __int_as_float(0x7fc00000);
-  const float ifx = __fdiv_rn(1.f, L.ffx), ify = __fdiv_rn(1.f, L.ffy);
+  const float ifx = L.fifx, ify = L.fify;
   // the front end's vertex, operation for operation
   auto vertex = [&](int x, int y, float z) {
     return make_float3(__fmul_rn(__fmul_rn(__fsub_rn((float)x, L.fcx), z), ifx),
@@ -590,17 +623,28 @@ cudaError_t launch_copy_frames(const FrameCopyList& list, int max_count, cudaStr
 
 cudaError_t launch_frontend(const DescList& list, int max_w, int max_h, int levels,
                             const KParams& P, cudaStream_t s) {
-  (void)levels;  // 1..4 levels and radius 0..4 (checked at tracker creation)
+  // 1..4 levels (the trackers' own) and radius 0..4: checked at tracker creation
   const dim3 blk(kTx, kTy);
   const dim3 g((max_w + kTile - 1) / kTile, (max_h + kTile - 1) / kTile, list.n);
-  const bool h = P.precision == KF_FP16;
+#define KF_FE(R, LV)                                                        \
+  (P.precision == KF_FP16 ? k_frontend_fused<__half, R, LV><<<g, blk, 0, s>>>(list, P) \
+                          : k_frontend_fused<float, R, LV><<<g, blk, 0, s>>>(list, P))
+  // the default radius has an instance for each number of levels
   switch (P.bil_radius) {
-    case 0: h ? k_frontend_fused<__half, 0><<<g, blk, 0, s>>>(list, P) : k_frontend_fused<float, 0><<<g, blk, 0, s>>>(list, P); break;
-    case 1: h ? k_frontend_fused<__half, 1><<<g, blk, 0, s>>>(list, P) : k_frontend_fused<float, 1><<<g, blk, 0, s>>>(list, P); break;
-    case 2: h ? k_frontend_fused<__half, 2><<<g, blk, 0, s>>>(list, P) : k_frontend_fused<float, 2><<<g, blk, 0, s>>>(list, P); break;
-    case 3: h ? k_frontend_fused<__half, 3><<<g, blk, 0, s>>>(list, P) : k_frontend_fused<float, 3><<<g, blk, 0, s>>>(list, P); break;
-    default: h ? k_frontend_fused<__half, 4><<<g, blk, 0, s>>>(list, P) : k_frontend_fused<float, 4><<<g, blk, 0, s>>>(list, P); break;
+    case 0: KF_FE(0, 0); break;
+    case 1: KF_FE(1, 0); break;
+    case 2:
+      switch (levels) {
+        case 1: KF_FE(2, 1); break;
+        case 2: KF_FE(2, 2); break;
+        case 3: KF_FE(2, 3); break;
+        default: KF_FE(2, 4); break;
+      }
+      break;
+    case 3: KF_FE(3, 0); break;
+    default: KF_FE(4, 0); break;
   }
+#undef KF_FE
   return cudaGetLastError();
 }
 

@@ -56,6 +56,7 @@ struct LevelMaps {
   int fw, fh;                 // frame level size
   int mw, mh;                 // model level size
   float ffx, ffy, fcx, fcy;   // frame level intrinsics (vertex map)
+  float fifx, fify;           // 1 / ffx and 1 / ffy, rounded once
   float mfx, mfy, mcx, mcy;   // model level intrinsics (projection)
   float* fdepth;              // filtered depth, fw * fh
   void* fA;                   // frame records, camera frame; vertex and normal NaN where
