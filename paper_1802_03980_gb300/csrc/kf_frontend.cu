@@ -229,6 +229,45 @@ __device__ __forceinline__ float bilateral_at(const float* s_raw, int RR, int cx
   return __fdividef(num, den);
 }
 
+// One frame by threads t0, t0 + stride, ...: over its 16-byte groups, kCopyU per
+// thread at a time (all loads issued before the stores); a source not on a
+// 16-byte boundary, and the last count % 4 floats, go one float at a time.
+constexpr int kCopyU = 4;
+__device__ __forceinline__ void copy_frame(const float* src, float* dst, int count, int t0, int stride) {
+  if ((reinterpret_cast<uintptr_t>(src) & 15u) == 0 && (reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
+    const int n4 = count / 4;
+    const float4* s4 = reinterpret_cast<const float4*>(src);
+    float4* d4 = reinterpret_cast<float4*>(dst);
+    for (int base = t0; base < n4; base += kCopyU * stride) {
+      float4 v[kCopyU];
+#pragma unroll
+      for (int u = 0; u < kCopyU; ++u) {
+        const int i = base + u * stride;
+        if (i < n4) v[u] = s4[i];
+      }
+#pragma unroll
+      for (int u = 0; u < kCopyU; ++u) {
+        const int i = base + u * stride;
+        if (i < n4) d4[i] = v[u];
+      }
+    }
+    for (int i = 4 * n4 + t0; i < count; i += stride) dst[i] = src[i];
+  } else {
+    for (int i = t0; i < count; i += stride) dst[i] = src[i];
+  }
+}
+
+// blockIdx.y: frame
+__global__ void __launch_bounds__(256) k_copy_frames(FrameCopyList list) {
+  const int f = blockIdx.y;
+  copy_frame(list.src[f], list.dst[f], list.count[f], blockIdx.x * blockDim.x + threadIdx.x,
+             gridDim.x * blockDim.x);
+}
+
+// Blocks of a front-end launch that copy the next launch's frames: 1.2 MB under
+// way, what the host link needs (200 GB/s), on a twelfth of the places.
+constexpr int kCopyBlocks = 76;
+
 // RB: the bilateral radius. kLv: the number of levels, or 0 for any (read from
 // the descriptor). What bounds a batch is instruction issue (78 % of the slots,
 // 476 instructions a level-0 pixel before the levels were known here, a third of
@@ -237,7 +276,8 @@ __device__ __forceinline__ float bilateral_at(const float* s_raw, int RR, int cx
 // and of the pyramid's means, and a bounds check and two stores a raw pixel.
 // Measured on GB300, 256 frames 640x480, three levels: 1217 -> 867 us.
 template <class T, int RB, int kLv>
-__global__ void __launch_bounds__(kTx* kTy, KF_FE_MINB) k_frontend_fused(DescList list, KParams P) {
+__global__ void __launch_bounds__(kTx* kTy, KF_FE_MINB) k_frontend_fused(DescList list, FrameCopyList next,
+                                                                            KParams P) {
   constexpr int r = RB;                                          // = P.bil_radius
   constexpr int kR0 = region0(kLv > 0 ? kLv : KF_MAX_LEVELS);    // largest of the instance
   constexpr int kRR = kR0 + 2 * r;
@@ -254,7 +294,17 @@ __global__ void __launch_bounds__(kTx* kTy, KF_FE_MINB) k_frontend_fused(DescLis
   __shared__ __align__(8) float s_d1[kR0 / 2 * (kR0 / 2)];
   __shared__ __align__(8) float s_d2[kR0 / 4 * (kR0 / 4)];
   __shared__ __align__(8) float s_d3[kR0 / 8 * (kR0 / 8)];
-  const PairDesc* d = list.d[blockIdx.z];
+  int z = blockIdx.z;
+  if (z < next.layers) {  // the grid's first layers copy
+    const int b = (z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    if (b < kCopyBlocks)
+      for (int f = 0; f < next.n; ++f)
+        copy_frame(next.src[f], next.dst[f], next.count[f], b * nthr + threadIdx.y * kTx + threadIdx.x,
+                   kCopyBlocks * nthr);
+    return;
+  }
+  z -= next.layers;
+  const PairDesc* d = list.d[z];
   const int W = d->iw, H = d->ih;
   const int X0 = blockIdx.x * kTile, Y0 = blockIdx.y * kTile;
   if (X0 >= W || Y0 >= H) return;
@@ -263,7 +313,7 @@ __global__ void __launch_bounds__(kTx* kTy, KF_FE_MINB) k_frontend_fused(DescLis
   const int RR = R0 + 2 * r;
   const int S = pair_stride(R0, RR);
   const int tid = threadIdx.y * kTx + threadIdx.x;
-  const float* D = list.depth[blockIdx.z];
+  const float* D = list.depth[z];
   // a thread loads a piece of a column, all of it before the first use: a pixel
   // is the lower half of its own pair and the upper half of the one above
   {
@@ -576,59 +626,30 @@ __global__ void __launch_bounds__(kTx * kTy) k_ii_normals(DescList list, IiGrid 
   }
 }
 
-// blockIdx.y: frame; threads stride over its 16-byte groups, kCopyU per
-// thread at a time (all loads issued before the stores); a source not on a
-// 16-byte boundary, and the last count % 4 floats, go one float at a time.
-constexpr int kCopyU = 4;
-__global__ void __launch_bounds__(256) k_copy_frames(FrameCopyList list) {
-  const int f = blockIdx.y;
-  const float* src = list.src[f];
-  float* dst = list.dst[f];
-  const int count = list.count[f];
-  const int stride = gridDim.x * blockDim.x;
-  const int t0 = blockIdx.x * blockDim.x + threadIdx.x;
-  if ((reinterpret_cast<uintptr_t>(src) & 15u) == 0 && (reinterpret_cast<uintptr_t>(dst) & 15u) == 0) {
-    const int n4 = count / 4;
-    const float4* s4 = reinterpret_cast<const float4*>(src);
-    float4* d4 = reinterpret_cast<float4*>(dst);
-    for (int base = t0; base < n4; base += kCopyU * stride) {
-      float4 v[kCopyU];
-#pragma unroll
-      for (int u = 0; u < kCopyU; ++u) {
-        const int i = base + u * stride;
-        if (i < n4) v[u] = s4[i];
-      }
-#pragma unroll
-      for (int u = 0; u < kCopyU; ++u) {
-        const int i = base + u * stride;
-        if (i < n4) d4[i] = v[u];
-      }
-    }
-    for (int i = 4 * n4 + t0; i < count; i += stride) dst[i] = src[i];
-  } else {
-    for (int i = t0; i < count; i += stride) dst[i] = src[i];
-  }
-}
-
 }  // namespace
 
-cudaError_t launch_copy_frames(const FrameCopyList& list, int max_count, cudaStream_t s) {
+cudaError_t launch_copy_frames(const FrameCopyList& list, cudaStream_t s) {
   if (list.n <= 0) return cudaSuccess;
+  int most = 0;
+  for (int i = 0; i < list.n; ++i) most = list.count[i] > most ? list.count[i] : most;
   const int per_block = 256 * 4 * kCopyU;  // floats per block per pass
-  int bx = (max_count + per_block - 1) / per_block;
+  int bx = (most + per_block - 1) / per_block;
   bx = bx < 1 ? 1 : (bx > 1024 ? 1024 : bx);
   k_copy_frames<<<dim3(bx, list.n), 256, 0, s>>>(list);
   return cudaGetLastError();
 }
 
-cudaError_t launch_frontend(const DescList& list, int max_w, int max_h, int levels,
+cudaError_t launch_frontend(const DescList& list, const FrameCopyList& pull, int max_w, int max_h, int levels,
                             const KParams& P, cudaStream_t s) {
   // 1..4 levels (the trackers' own) and radius 0..4: checked at tracker creation
   const dim3 blk(kTx, kTy);
-  const dim3 g((max_w + kTile - 1) / kTile, (max_h + kTile - 1) / kTile, list.n);
+  const int tx = (max_w + kTile - 1) / kTile, ty = (max_h + kTile - 1) / kTile;
+  FrameCopyList next = pull;
+  next.layers = next.n > 0 ? (kCopyBlocks + tx * ty - 1) / (tx * ty) : 0;
+  const dim3 g(tx, ty, list.n + next.layers);
 #define KF_FE(R, LV)                                                        \
-  (P.precision == KF_FP16 ? k_frontend_fused<__half, R, LV><<<g, blk, 0, s>>>(list, P) \
-                          : k_frontend_fused<float, R, LV><<<g, blk, 0, s>>>(list, P))
+  (P.precision == KF_FP16 ? k_frontend_fused<__half, R, LV><<<g, blk, 0, s>>>(list, next, P) \
+                          : k_frontend_fused<float, R, LV><<<g, blk, 0, s>>>(list, next, P))
   // the default radius has an instance for each number of levels
   switch (P.bil_radius) {
     case 0: KF_FE(0, 0); break;

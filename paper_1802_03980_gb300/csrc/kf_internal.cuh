@@ -299,14 +299,19 @@ namespace kf {
 // Frames of a batch pulled from page-locked host memory into device buffers
 // by one kernel (16-byte loads, several in flight per thread), instead of
 // one copy per frame issued by the host.
+constexpr int kPullMax = 32;                 // page-locked host frames per launch, and the
+constexpr long long kPullPixels = 1200000;   // pixels from which on a launch takes no more
 struct FrameCopyList {
-  const float* src[kDescListMax];
-  float* dst[kDescListMax];
-  int count[kDescListMax];  // floats
+  const float* src[kPullMax];
+  float* dst[kPullMax];
+  int count[kPullMax];  // floats
   int n;
+  int layers;           // of the front end's grid (launch_frontend)
 };
-cudaError_t launch_copy_frames(const FrameCopyList& list, int max_count, cudaStream_t s);
-cudaError_t launch_frontend(const DescList& list, int max_w, int max_h, int levels,
+cudaError_t launch_copy_frames(const FrameCopyList& list, cudaStream_t s);
+// next: page-locked host frames of a later launch, copied by a few of this one's
+// blocks meanwhile
+cudaError_t launch_frontend(const DescList& list, const FrameCopyList& next, int max_w, int max_h, int levels,
                             const KParams& P, cudaStream_t s);
 // integral-image normals of every level of the listed frames (after the
 // front end): replaces the frame normals and drops vertices without one
