@@ -393,6 +393,8 @@ __global__ void __launch_bounds__(128) k_raycast(const float2* FW, VolGeom g, Ne
   // the sample before k: known (have: observed, with value fp at depth zp) or leapt over
   bool known = true, have = false;
   float zp = 0.f, fp = 0.f;
+  bool hit = false;
+  float fh = 0.f;  // the value behind the surface
   for (int k = 0; k < rp.steps;) {
     const float z = depth_of(k);
     if (z > rp.zf) break;
@@ -430,30 +432,8 @@ __global__ void __launch_bounds__(128) k_raycast(const float2* FW, VolGeom g, Ne
       known = true;
     }
     if (known && have && fp > 0.f && f <= 0.f) {
-      const float zs = __fadd_rn(zp, __fmul_rn(rp.dz, __fdiv_rn(fp, __fsub_rn(fp, f))));
-      const float vx = __fadd_rn(rp.c[0], __fmul_rn(zs, dx));
-      const float vy = __fadd_rn(rp.c[1], __fmul_rn(zs, dy));
-      const float vz = __fadd_rn(rp.c[2], __fmul_rn(zs, dzv));
-      float a[3], b[3];
-      bool ok = sample<kAny>(FW, g, rp.rs, __fadd_rn(vx, g.s), vy, vz, a[0]);
-      ok = sample<kAny>(FW, g, rp.rs, __fsub_rn(vx, g.s), vy, vz, b[0]) && ok;
-      ok = sample<kAny>(FW, g, rp.rs, vx, __fadd_rn(vy, g.s), vz, a[1]) && ok;
-      ok = sample<kAny>(FW, g, rp.rs, vx, __fsub_rn(vy, g.s), vz, b[1]) && ok;
-      ok = sample<kAny>(FW, g, rp.rs, vx, vy, __fadd_rn(vz, g.s), a[2]) && ok;
-      ok = sample<kAny>(FW, g, rp.rs, vx, vy, __fsub_rn(vz, g.s), b[2]) && ok;
-      if (ok) {
-        const float gx = a[0] - b[0], gy = a[1] - b[1], gz = a[2] - b[2];
-        const float n2 = gx * gx + gy * gy + gz * gz;
-        if (n2 > 0.f) {
-          const float inv = 1.f / sqrtf(n2);
-          out[0] = vx;
-          out[1] = vy;
-          out[2] = vz;
-          out[3] = gx * inv;
-          out[4] = gy * inv;
-          out[5] = gz * inv;
-        }
-      }
+      hit = true;
+      fh = f;
       break;
     }
     if (known && have && fp < 0.f && f > 0.f) break;  // a back face: no surface
@@ -461,6 +441,36 @@ __global__ void __launch_bounds__(128) k_raycast(const float2* FW, VolGeom g, Ne
     zp = z;
     fp = f;
     ++k;
+  }
+  // the normals' samples once for all rays of the warp, wherever each met its
+  // surface: inside the loop they ran for each sample at which some ray met it (map
+  // and raycast at 512^3 and 640x480: 100 -> 96 us)
+  __syncwarp();
+  if (hit) {
+    const float zs = __fadd_rn(zp, __fmul_rn(rp.dz, __fdiv_rn(fp, __fsub_rn(fp, fh))));
+    const float vx = __fadd_rn(rp.c[0], __fmul_rn(zs, dx));
+    const float vy = __fadd_rn(rp.c[1], __fmul_rn(zs, dy));
+    const float vz = __fadd_rn(rp.c[2], __fmul_rn(zs, dzv));
+    float a[3], b[3];
+    bool ok = sample<kAny>(FW, g, rp.rs, __fadd_rn(vx, g.s), vy, vz, a[0]);
+    ok = sample<kAny>(FW, g, rp.rs, __fsub_rn(vx, g.s), vy, vz, b[0]) && ok;
+    ok = sample<kAny>(FW, g, rp.rs, vx, __fadd_rn(vy, g.s), vz, a[1]) && ok;
+    ok = sample<kAny>(FW, g, rp.rs, vx, __fsub_rn(vy, g.s), vz, b[1]) && ok;
+    ok = sample<kAny>(FW, g, rp.rs, vx, vy, __fadd_rn(vz, g.s), a[2]) && ok;
+    ok = sample<kAny>(FW, g, rp.rs, vx, vy, __fsub_rn(vz, g.s), b[2]) && ok;
+    if (ok) {
+      const float gx = a[0] - b[0], gy = a[1] - b[1], gz = a[2] - b[2];
+      const float n2 = gx * gx + gy * gy + gz * gz;
+      if (n2 > 0.f) {
+        const float inv = 1.f / sqrtf(n2);
+        out[0] = vx;
+        out[1] = vy;
+        out[2] = vz;
+        out[3] = gx * inv;
+        out[4] = gy * inv;
+        out[5] = gz * inv;
+      }
+    }
   }
   const size_t p = ((size_t)v * cam.w + u) * 3;
   V[p] = out[0];
