@@ -47,6 +47,10 @@ namespace {
 constexpr int kTeamWarps = 4;            // item warps of a half item
 constexpr int kTeamBlock = 2 * 32 * kTeamWarps;  // two warps (parts) for each
 constexpr int kPollCheck = 64;  // polls between two looks at the clock
+// pause between two polls of a worker without half items at its level
+#ifndef KF_TEAM_IDLE_NS
+#define KF_TEAM_IDLE_NS 100
+#endif
 
 __device__ __forceinline__ void packet_store(unsigned long long* p, unsigned v, unsigned tag) {
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(((unsigned long long)tag << 32) | v)
@@ -153,6 +157,7 @@ struct TeamShared {
   ItemSumWord part[kBlockWarps][kSums];
   double sums[kSums + 3];
   int level, w0, w1;
+  unsigned it;
   int N, kmed, klo, khi, hit, stop;
   unsigned matched;
   int abort;
@@ -296,14 +301,19 @@ __device__ __forceinline__ void flush_hist(unsigned* sh_hist, unsigned* hist, in
   }
 }
 
-// A worker: the half items w, w + W, ... of the pair's current level.
+// A worker: the half items w, w + W, ... of the pair's current level. The leader
+// waits for the sums of the workers that have some, so such a worker meets every
+// message; one without may sleep through a whole iteration (its block started
+// late, say) and goes on from the first message that it finds complete, the
+// iteration's number taken from the tag.
 template <class T, int kA>
 __device__ void team_work(const PairDesc* d, const TeamPair& tp, int w, unsigned long long limit_ns,
                           const KParams& P, TeamShared& sh, unsigned* sh_hist) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int lw = warp % kTeamWarps, part = warp / kTeamWarps;
   int level = P.levels - 1, w0 = -1, w1 = -1;
-  for (unsigned it = 0;; ++it) {
+  unsigned it = 0;
+  for (;;) {
     const LevelMaps L = d->lv[level];
     const int chunk = level_chunk(level), fn = L.fw * L.fh;
     const int halves = 2 * ((fn + chunk - 1) / chunk);
@@ -377,22 +387,27 @@ __device__ void team_work(const PairDesc* d, const TeamPair& tp, int w, unsigned
     if (warp == 0) {
       Wait wait;
       unsigned long long v;
+      unsigned ahead;  // iterations; an earlier launch's tag lies far beyond kTeamTags
       bool ok = true;
       for (;;) {
         v = packet_load(d->team_msg + lane);
-        if (__all_sync(0xffffffffu, (unsigned)(v >> 32) == tp.tag + it + 1u)) break;
+        ahead = (unsigned)(v >> 32) - (tp.tag + it);
+        const bool same = ahead == __shfl_sync(0xffffffffu, ahead, 0);
+        if (__all_sync(0xffffffffu, same && ahead - 1u < kTeamTags - 1u)) break;
         if (__any_sync(0xffffffffu, wait.ran_out(limit_ns))) {
           ok = false;
           break;
         }
-        if (w >= halves) __nanosleep(100);  // nothing to do at this level
+        if (w >= halves) __nanosleep(KF_TEAM_IDLE_NS);  // nothing to do at this level
       }
       if (lane < 24) sh.xf[lane] = __uint_as_float((unsigned)v);
       if (lane == 24) sh.level = ok ? (int)(unsigned)v : -1;
+      if (lane == 24) sh.it = it + ahead;
       if (lane == 25) sh.w0 = (int)(unsigned)v;
       if (lane == 26) sh.w1 = (int)(unsigned)v;
     }
     __syncthreads();
+    it = sh.it;
     level = sh.level;
     w0 = sh.w0;
     w1 = sh.w1;
