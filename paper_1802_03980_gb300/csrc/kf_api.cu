@@ -697,7 +697,7 @@ kf_status kf_track_create(const kf_params* p, int max_w, int max_h, void* cuda_s
     part(&t->d_dbg_pose, sizeof(double) * 16);
     if (team) {
       const size_t first = at;
-      part(&D.team_hist, sizeof(unsigned) * 3 * team_hist_words(p->hist_bins));
+      part(&D.team_hist, sizeof(unsigned) * kTeamHists * team_hist_words(p->hist_bins));
       part(&D.team_msg, 32 * sizeof(unsigned long long));
       part(&D.team_rows, (size_t)t->max_items * 2 * 32 * sizeof(unsigned long long));
       t->d_team = D.team_hist;

@@ -111,10 +111,10 @@ struct PairDesc {
                               // warp w of item li packs its records from place
                               // li * chunk + w * chunk / kBlockWarps
   unsigned* wcount;           // [items * kBlockWarps] records per item and warp
-  // team launch (null when the tracker's frames are too large for it): three
-  // rotating histograms, the leader's message and the half items' sums (packets
+  // team launch (null when the tracker's frames are too large for it): rotating
+  // histograms, the leader's message and the half items' sums (packets
   // of a value and its tag), all zero between launches but for the packets
-  unsigned* team_hist;        // [3 * team_hist_words(bins)]
+  unsigned* team_hist;        // [kTeamHists * team_hist_words(bins)]
   unsigned long long* team_msg;   // [32]
   unsigned long long* team_rows;  // [2 * items * 32]
   int* dbg_index;             // [iw*ih] inspection outputs (may be null)
@@ -147,6 +147,9 @@ constexpr int kMaxSchedPairs = 65535;      // 16-bit pair field
 // take, pairs of a launch.
 __host__ __device__ constexpr int team_hist_none(int bins) { return (bins + 3) / 4 * 4; }
 __host__ __device__ constexpr int team_hist_words(int bins) { return team_hist_none(bins) + 4; }
+constexpr unsigned kTeamHists = 16;   // rotating histograms, a power of two
+constexpr unsigned kTeamAcquire = 8;  // iterations between two acquires, a power of two
+static_assert(kTeamHists >= kTeamAcquire + 1 + 2, "a clear comes before the messages of two iterations on");
 constexpr int kTeamSlots = 8;
 constexpr int kTeamMaxItems = 1024;  // items of the largest frame
 constexpr int kTeamMaxPairs = 16;

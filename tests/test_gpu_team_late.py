@@ -4,7 +4,9 @@ A worker without half items at the pair's level only waits for the next
 message, and the leader does not wait for it, so it may sleep through messages
 and has to go on from the one it finds. A build whose idle workers sleep some
 60 us between two looks (an iteration takes about 9) misses several in every
-alignment: the same bits as the ordinary build's, and no time-out.
+alignment: the same bits as the ordinary build's, and no time-out. The last
+case runs more iterations than there are rotating histograms; its bits are also
+those of the launches per iteration, which have none.
 """
 import json
 import os
@@ -21,9 +23,10 @@ pytestmark = pytest.mark.gpu
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
-# batches whose coarse levels leave workers without items
-CASES = [([(640, 480)], 3, (10, 5, 4)), ([(1280, 960)], 4, (4, 3, 3, 2)),
-         ([(640, 480), (333, 251), (160, 120)], 3, (10, 5, 4))]
+# batches whose coarse levels leave workers without items; flags
+CASES = [([(640, 480)], 3, (10, 5, 4), 7), ([(1280, 960)], 4, (4, 3, 3, 2), 7),
+         ([(640, 480), (333, 251), (160, 120)], 3, (10, 5, 4), 7),
+         ([(640, 480), (160, 120)], 3, (19, 9, 11), 3)]
 
 CHILD = r"""
 import json, sys
@@ -33,11 +36,11 @@ print("RESULT " + json.dumps(alignments()))
 """
 
 
-def alignments():
+def alignments(cases=CASES):
     k = H.kf()
     out = []
-    for sizes, levels, caps in CASES:
-        p, _ = H.params(levels=levels, caps=caps)
+    for sizes, levels, caps, flags in cases:
+        p, _ = H.params(levels=levels, caps=caps, flags=flags)
         pairs = [S.config2_kinect(60 + i, *sz) for i, sz in enumerate(sizes)]
         trk = [H.Tracker(p, *sz) for sz in sizes]
         try:
@@ -66,3 +69,6 @@ def test_workers_that_sleep_through_messages_change_no_bit(tmp_path):
     assert r.returncode == 0, r.stderr[-2000:]
     late = json.loads([x for x in r.stdout.splitlines() if x.startswith("RESULT ")][-1][len("RESULT "):])
     assert late == alignments()
+    sizes, levels, caps, flags = CASES[-1]
+    general = alignments([(sizes, levels, caps, flags | H.kf().KF_LAUNCH_PER_ITERATION)])
+    assert late[-8:] == general
