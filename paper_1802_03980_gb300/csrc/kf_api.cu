@@ -359,6 +359,7 @@ bool plan_teams(kf_tracker* const* trk, Plan* pl) {
     TeamPair& tp = pl->args.pair[k];
     tp.d = trk[pl->order[k]]->d_desc;
     tp.first = pl->grid;
+    tp.slots = slots;
     tp.workers = (halves[k] + slots - 1) / slots;
     pl->grid += 1 + tp.workers;
   }
@@ -676,9 +677,12 @@ kf_status kf_track_create(const kf_params* p, int max_w, int max_h, void* cuda_s
   t->max_items = (int)((px0 + kChunk - 1) / kChunk);
   D.partial_cap = t->max_items;
   D.px_cap = (int)px0;
+  // an item's places, and a chunk of padding for the first reads (fix_issue); a
+  // team's workers have room for whole slots: less than kTeamSlots half items more
+  const bool team = t->max_items <= kTeamMaxItems;
+  D.rec_cap = (int)std::max(px0 + kChunk, team ? (size_t)(2 * t->max_items + kTeamSlots) * (kChunk / 2) : 0);
   // two allocations, cut into 256-byte aligned parts: what starts at zero, and
   // the maps (an allocation each made creation mostly allocation calls)
-  const bool team = t->max_items <= kTeamMaxItems;
   char* base = nullptr;
   size_t at = 0;
   auto part = [&](auto** ptr, size_t bytes) {
@@ -718,7 +722,7 @@ kf_status kf_track_create(const kf_params* p, int max_w, int max_h, void* cuda_s
     }
     part(&D.partials, sizeof(float) * kPartialStride * t->max_items);
     part(&D.wcount, sizeof(unsigned) * kBlockWarps * t->max_items);
-    part(&D.recs, 2 * sizeof(float4) * (px0 + kChunk));
+    part(&D.recs, 2 * sizeof(float4) * (size_t)D.rec_cap);
   };
   maps();  // sizes first, then the parts' addresses
   if ((e = tmalloc(t, &base, at)) != cudaSuccess) return bail(e);

@@ -105,11 +105,12 @@ struct PairDesc {
   unsigned* hist;             // [bins]
   float* partials;            // [items][kPartialStride]
   unsigned* counters;         // [2]: histogram stage, reduction stage
-  float4* recs;               // [2 * (px + kChunk)] records of the window pixels:
+  float4* recs;               // [2 * rec_cap] records of the window pixels:
                               // row a[0..5], b and bin (int bits), written by the
                               // association pass, read by the reduction pass;
                               // warp w of item li packs its records from place
-                              // li * chunk + w * chunk / kBlockWarps
+                              // li * chunk + w * chunk / kBlockWarps (in a team
+                              // launch a block's are its own, see TeamPair)
   unsigned* wcount;           // [items * kBlockWarps] records per item and warp
   // team launch (null when the tracker's frames are too large for it): rotating
   // histograms, the leader's message and the half items' sums (packets
@@ -120,7 +121,9 @@ struct PairDesc {
   int* dbg_index;             // [iw*ih] inspection outputs (may be null)
   int* dbg_bin;
   int partial_cap;            // work-item partials the buffer holds
-  int px_cap;                 // frame pixels recs (+ kChunk) / dbg_* hold
+  int px_cap;                 // frame pixels dbg_* hold
+  int rec_cap;                // record places
+  int pad_;
 };
 
 // Active work list of one launch, built on the device (int buffer):
@@ -151,6 +154,7 @@ constexpr unsigned kTeamHists = 16;   // rotating histograms, a power of two
 constexpr unsigned kTeamAcquire = 8;  // iterations between two acquires, a power of two
 static_assert(kTeamHists >= kTeamAcquire + 1 + 2, "a clear comes before the messages of two iterations on");
 constexpr int kTeamSlots = 8;
+constexpr int kTeamPlaces = level_chunk(0) / kBlockWarps;  // record places of an item warp, at any level
 constexpr int kTeamMaxItems = 1024;  // items of the largest frame
 constexpr int kTeamMaxPairs = 16;
 
@@ -214,13 +218,14 @@ struct PairInput {
 struct PairOutput;
 
 // One pair of a team launch: its blocks are [first, first + 1 + workers), the
-// first its leader. tag: distinguishes this launch's packets from all earlier
+// first its leader; a worker takes up to `slots` half items, worker w's records
+// of the s-th at places (w slots + s) 4 kTeamPlaces on. tag: distinguishes this launch's packets from all earlier
 // ones (plus an iteration's number, below kTeamTags).
 struct TeamPair {
   const PairDesc* d;
   PairOutput* out;
   unsigned tag;
-  int first, workers;
+  int first, workers, slots;
 };
 constexpr unsigned kTeamTags = 4096;  // > the iterations of an alignment + 1
 

@@ -52,6 +52,7 @@ void checked_fault_team(long long out[3]) { take_fault(out); }
 namespace {
 
 constexpr int kTeamWarps = 4;            // item warps of a half item
+static_assert(kTeamWarps * kTeamPlaces == level_chunk(0) / 2, "record places of a half item");
 constexpr int kTeamBlock = 2 * 32 * kTeamWarps;  // two warps (parts) for each
 constexpr int kPollCheck = 64;  // polls between two looks at the clock
 // pause between two polls of a worker without half items at its level
@@ -178,13 +179,15 @@ struct TeamShared {
 // two, part 0 takes the first half and part 1 the second. Each looks up, counts
 // and forms the rows of its kN pixels at the same time; only the additions stay
 // in order: part 0 hands its lanes' sums to part 1, which goes on from them and
-// writes the warp's row. Part 1's records start half a region on (fix_place).
+// writes the warp's row. places: the first of the item warp's records, in the
+// block's own part of the buffer: no other block of the launch, at this level or
+// the next, writes or reads there. Part 1's start half the item warp's pixels on.
 // Alone on its scheduler a warp took 5.9 us for the 16 pixels a lane has at level
 // 0 (640x480), two take 3.6 us.
 template <class T, int kA, int kPass, int kN>
 __device__ __forceinline__ void team_batch(const PairDesc* d, const LevelMaps& L, int li, int vw, int lw,
                                            int part, int chunk, const KParams& P, TeamShared& sh, int s,
-                                           unsigned* sh_hist, int lo, int hi, float* row) {
+                                           unsigned* sh_hist, int lo, int hi, int places, float* row) {
   const int lane = threadIdx.x & 31, t = vw * 32 + lane;
   const int ib = li * chunk, b0 = ib + part * kN * kBlock;
   const int e = min(min(L.fw * L.fh, ib + chunk), b0 + kN * kBlock);
@@ -198,7 +201,7 @@ __device__ __forceinline__ void team_batch(const PairDesc* d, const LevelMaps& L
     float sum[kSumRegs];
     float (*hand)[32] = sh.hand[s & 1][lw];
     int wc = 0;
-    const int rbase = ib + vw * (chunk / kBlockWarps) + part * (chunk / kBlockWarps / 2);
+    const int rbase = places + part * (chunk / kBlockWarps / 2);
     if (part == 0) {
       zero_sums(sum);
       finish_rows<kA, kPass, kN>(d, b, bin, lo, hi, sum, rbase, wc);
@@ -220,16 +223,16 @@ __device__ __forceinline__ void team_batch(const PairDesc* d, const LevelMaps& L
 template <class T, int kA, int kPass>
 __device__ __noinline__ void team_item(const PairDesc* d, const LevelMaps& maps, int li, int vw, int lw,
                                        int part, int chunk, const KParams& P, TeamShared& sh, int s,
-                                       unsigned* sh_hist, int lo, int hi, float* row) {
+                                       unsigned* sh_hist, int lo, int hi, int places, float* row) {
   const LevelMaps L = maps;  // in registers: the caller's copy lies in its stack frame
   static_assert(level_chunk(0) == 16 * kBlock && level_chunk(1) == 8 * kBlock && level_chunk(2) == 4 * kBlock &&
                     level_chunk(3) == 4 * kBlock, "pixels of a lane per level");
   if (chunk == 16 * kBlock)
-    team_batch<T, kA, kPass, 8>(d, L, li, vw, lw, part, chunk, P, sh, s, sh_hist, lo, hi, row);
+    team_batch<T, kA, kPass, 8>(d, L, li, vw, lw, part, chunk, P, sh, s, sh_hist, lo, hi, places, row);
   else if (chunk == 8 * kBlock)
-    team_batch<T, kA, kPass, 4>(d, L, li, vw, lw, part, chunk, P, sh, s, sh_hist, lo, hi, row);
+    team_batch<T, kA, kPass, 4>(d, L, li, vw, lw, part, chunk, P, sh, s, sh_hist, lo, hi, places, row);
   else
-    team_batch<T, kA, kPass, 2>(d, L, li, vw, lw, part, chunk, P, sh, s, sh_hist, lo, hi, row);
+    team_batch<T, kA, kPass, 2>(d, L, li, vw, lw, part, chunk, P, sh, s, sh_hist, lo, hi, places, row);
 }
 
 // The recorded rows of one item warp with klo <= bin <= khi, added in packed
@@ -244,15 +247,17 @@ struct TeamFix {
       const int i = e0 + r * 32 + (threadIdx.x & 31);
       if (i < total) {
         const size_t at = base + (i < c0 ? i : half + i - c0);
-        r0[r] = __ldcg(d->recs + 2 * at);
-        r1[r] = __ldcg(d->recs + 2 * at + 1);
+        KF_GUARD((int)at < d->rec_cap, 12, (int)at, d->rec_cap) {
+          r0[r] = __ldcg(d->recs + 2 * at);
+          r1[r] = __ldcg(d->recs + 2 * at + 1);
+        }
       }
     }
   }
-  __device__ __forceinline__ void begin(const PairDesc* d, int li, int vw, int chunk, const int (&count)[2]) {
+  __device__ __forceinline__ void begin(const PairDesc* d, int places, int chunk, const int (&count)[2]) {
     c0 = count[0];
     total = c0 + count[1];
-    base = li * chunk + vw * (chunk / kBlockWarps);
+    base = places;
     half = chunk / kBlockWarps / 2;
     issue(d, 0);
   }
@@ -323,6 +328,8 @@ __device__ void team_work(const PairDesc* d, const TeamPair& tp, int w, unsigned
   const int lw = warp % kTeamWarps, part = warp / kTeamWarps;
   int level = P.levels - 1, w0 = -1, w1 = -1;
   unsigned it = 0;
+  // first record place of a slot's item warp
+  auto places_of = [&](int slot) { return ((w * tp.slots + slot) * kTeamWarps + lw) * kTeamPlaces; };
   for (;;) {
     const LevelMaps L = d->lv[level];
     const int chunk = level_chunk(level), fn = L.fw * L.fh;
@@ -339,9 +346,10 @@ __device__ void team_work(const PairDesc* d, const TeamPair& tp, int w, unsigned
           for (int k = 0; k < kTeamWarps; ++k)
             pixels += ip / kBlock * 32 + min(32, max(0, rest - ((hid & 1) + 2 * k) * 32));
         if (w0 >= 0)
-          team_item<T, kA, kPassSplit>(d, L, li, vw, lw, part, chunk, P, sh, s, sh_hist, w0, w1, sh.row_a[s][lw]);
+          team_item<T, kA, kPassSplit>(d, L, li, vw, lw, part, chunk, P, sh, s, sh_hist, w0, w1, places_of(s),
+                                       sh.row_a[s][lw]);
         else
-          team_item<T, kA, kPassHist>(d, L, li, vw, lw, part, chunk, P, sh, s, sh_hist, 0, 0, nullptr);
+          team_item<T, kA, kPassHist>(d, L, li, vw, lw, part, chunk, P, sh, s, sh_hist, 0, 0, 0, nullptr);
       }
       const int slots = s;
       __syncthreads();
@@ -351,7 +359,7 @@ __device__ void team_work(const PairDesc* d, const TeamPair& tp, int w, unsigned
       TeamFix f;
       auto item_of = [&](int slot) { return (w + slot * tp.workers) >> 1; };
       auto warp_of = [&](int slot) { return ((w + slot * tp.workers) & 1) + 2 * lw; };
-      if (w0 >= 0 && part < slots) f.begin(d, item_of(part), warp_of(part), chunk, sh.count[part][lw]);
+      if (w0 >= 0 && part < slots) f.begin(d, places_of(part), chunk, sh.count[part][lw]);
       if (warp == 0) {
         int N, kmed;
         const bool ok = warp_median(hist, P.bins, (unsigned)fn, limit_ns, N, kmed);
@@ -370,7 +378,7 @@ __device__ void team_work(const PairDesc* d, const TeamPair& tp, int w, unsigned
           if (hit) {
             s = s0 + part;
             if (s < slots) {
-              if (s0 > 0) f.begin(d, item_of(s), warp_of(s), chunk, sh.count[s][lw]);
+              if (s0 > 0) f.begin(d, places_of(s), chunk, sh.count[s][lw]);
               const float r = f.finish(d, klo, khi);
               if (lane < kSums) sh.row[part][lw][lane] = __fadd_rn(sh.row_a[s][lw][lane], r);
             }
@@ -378,7 +386,7 @@ __device__ void team_work(const PairDesc* d, const TeamPair& tp, int w, unsigned
             for (s = s0; s < min(s0 + 2, slots); ++s) {
               float* row = sh.row[s & 1][lw];
               team_item<T, kA, kPassBand>(d, L, item_of(s), warp_of(s), lw, part, chunk, P, sh, s, nullptr, klo,
-                                          khi, row);
+                                          khi, 0, row);
               if (part == 1 && lane < kSums) row[lane] = __fadd_rn(0.f, row[lane]);
             }
           }
@@ -388,7 +396,9 @@ __device__ void team_work(const PairDesc* d, const TeamPair& tp, int w, unsigned
           if (lw == 0 && s < slots && lane < kSums) {
             float (*r)[32] = sh.row[part];
             const float v = __fadd_rn(__fadd_rn(r[0][lane], r[2][lane]), __fadd_rn(r[1][lane], r[3][lane]));
-            packet_store(d->team_rows + (size_t)(w + s * tp.workers) * 32 + lane, __float_as_uint(v), tp.tag + it);
+            const int half = w + s * tp.workers;
+            KF_GUARD(half < 2 * d->partial_cap, 13, half, d->partial_cap)
+            packet_store(d->team_rows + (size_t)half * 32 + lane, __float_as_uint(v), tp.tag + it);
           }
           if (s0 + 2 < slots) __syncthreads();  // the rows are free again
         }
