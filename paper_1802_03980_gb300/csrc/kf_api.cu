@@ -231,7 +231,7 @@ cudaError_t tmalloc(kf_tracker* t, T** p, size_t bytes) {
 
 // Grid sizes of the tracker's launches: occupancy queries, asked once per device
 // and kernel variant (a batch creates its trackers one after the other).
-void launch_sizes(kf_tracker* t) {
+cudaError_t launch_sizes(kf_tracker* t) {
   struct Sizes {
     int device, precision, angle, shoot, bins;
     int assoc, reduce, sched, team;
@@ -239,7 +239,8 @@ void launch_sizes(kf_tracker* t) {
   static std::mutex mutex;
   static std::vector<Sizes> known;
   const KParams& P = t->kp;
-  icp_attributes(P);
+  const cudaError_t e = icp_attributes(P);
+  if (e != cudaSuccess) return e;
   std::lock_guard<std::mutex> lock(mutex);
   auto it = std::find_if(known.begin(), known.end(), [&](const Sizes& s) {
     return s.device == t->device && s.precision == P.precision && s.angle == P.use_angle &&
@@ -255,6 +256,7 @@ void launch_sizes(kf_tracker* t) {
   t->grid_reduce = it->reduce;
   t->grid_sched = it->sched;
   t->team_blocks = it->team;
+  return cudaSuccess;
 }
 
 bool intr_valid(const kf_intrinsics* K, int levels, int max_w, int max_h, std::string& why) {
@@ -734,7 +736,7 @@ kf_status kf_track_create(const kf_params* p, int max_w, int max_h, void* cuda_s
   zeroed();
   if ((e = cudaMemsetAsync(base, 0, zero_bytes, t->stream)) != cudaSuccess) return bail(e);
   D.depth_raw = t->d_depth_raw;
-  launch_sizes(t);
+  if ((e = launch_sizes(t)) != cudaSuccess) return bail(e);
   D.st = t->d_state;
   if ((e = cudaMemcpyAsync(t->d_desc, &D, sizeof(PairDesc), cudaMemcpyHostToDevice, t->stream)) != cudaSuccess) return bail(e);
   const PairDesc* self = t->d_desc;

@@ -288,8 +288,8 @@ __device__ void assoc_items(const PairDesc* d, const LevelMaps& L, int first, in
 constexpr int kRingU = KF_RING_U;  // pixels of a thread per batch
 static_assert(level_chunk(KF_MAX_LEVELS - 1) % (kRingU * kBlock) == 0, "a batch lies in one item");
 // bytes of the block's histogram, rounded up for what follows it
-__host__ __device__ __forceinline__ size_t hist_bytes(const KParams& P) {
-  return ((size_t)P.bins * sizeof(unsigned) + 15) / 16 * 16;
+__host__ __device__ __forceinline__ size_t hist_bytes(int bins) {
+  return ((size_t)bins * sizeof(unsigned) + 15) / 16 * 16;
 }
 #ifndef KF_RING_AHEAD
 #define KF_RING_AHEAD 1
@@ -931,7 +931,7 @@ __global__ void __launch_bounds__(kBlock, KF_SCHED_MINB) k_icp_sched(const PairD
                                                                      KParams P) {
   extern __shared__ __align__(16) unsigned char sh_raw[];
   unsigned* sh_hist = reinterpret_cast<unsigned*>(sh_raw);
-  [[maybe_unused]] Ring<T>* ring = reinterpret_cast<Ring<T>*>(sh_raw + hist_bytes(P));
+  [[maybe_unused]] Ring<T>* ring = reinterpret_cast<Ring<T>*>(sh_raw + hist_bytes(P.bins));
   __shared__ __align__(16) float sxf[24];  // 16-byte vector loads (load_xf)
   __shared__ unsigned long long s_word;
   __shared__ int s_last, s_flag, s_a, s_b, s_hit;
@@ -1067,7 +1067,7 @@ __global__ void __launch_bounds__(kBlock, KF_SCHED_MINB) k_icp_sched(const PairD
 
 // the block's histogram, and the ring of the variants that have one
 template <class T, int kA>
-size_t sched_smem(const KParams& P) { return hist_bytes(P) + (kA == 0 ? sizeof(Ring<T>) : 0); }
+size_t sched_smem(int bins) { return hist_bytes(bins) + (kA == 0 ? sizeof(Ring<T>) : 0); }
 
 template <class K>
 int wave(K kernel, size_t smem) {
@@ -1080,14 +1080,17 @@ int wave(K kernel, size_t smem) {
 
 }  // namespace
 
-void icp_attributes(const KParams& P) {
-  const int sm = P.bins * (int)sizeof(unsigned);
-#define KF_X(T, A)                                                                               \
-  cudaFuncSetAttribute(k_assoc_hist<T, A>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm); \
-  cudaFuncSetAttribute(k_icp_sched<T, A>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sched_smem<T, A>(P))
+cudaError_t icp_attributes(const KParams& P) {
+  const int sm = kMaxBins * (int)sizeof(unsigned);
+  cudaError_t e = cudaSuccess;
+#define KF_X(T, A)                                                                                     \
+  e = cudaFuncSetAttribute(k_assoc_hist<T, A>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);       \
+  if (e == cudaSuccess)                                                                                \
+    e = cudaFuncSetAttribute(k_icp_sched<T, A>, cudaFuncAttributeMaxDynamicSharedMemorySize,           \
+                             (int)sched_smem<T, A>(kMaxBins))
   KF_ASSOC_SWITCH(P, KF_X);
 #undef KF_X
-  team_attributes(P);
+  return e == cudaSuccess ? team_attributes(P) : e;
 }
 
 void icp_grids(const KParams& P, int* g_assoc, int* g_reduce, int* g_sched) {
@@ -1095,7 +1098,7 @@ void icp_grids(const KParams& P, int* g_assoc, int* g_reduce, int* g_sched) {
 #define KF_X(T, A)                                 \
   *g_assoc = wave(k_assoc_hist<T, A>, sm);         \
   *g_reduce = wave(k_reduce_solve<T, A>, 0);       \
-  *g_sched = wave(k_icp_sched<T, A>, sched_smem<T, A>(P))
+  *g_sched = wave(k_icp_sched<T, A>, sched_smem<T, A>(P.bins))
   KF_ASSOC_SWITCH(P, KF_X);
 #undef KF_X
   // one partition of the items for both passes
@@ -1107,7 +1110,7 @@ cudaError_t launch_icp_sched(const PairDesc* const* descs, const PairInput* in, 
                              unsigned long long wait_limit_ns, const KParams& P, cudaStream_t s) {
   unsigned long long* slots = reinterpret_cast<unsigned long long*>(queue + kQHeaderWords);
 #define KF_X(T, A) \
-  k_icp_sched<T, A><<<grid, kBlock, sched_smem<T, A>(P), s>>>(descs, in, out, n, queue, slots, qmask, wait_limit_ns, P)
+  k_icp_sched<T, A><<<grid, kBlock, sched_smem<T, A>(P.bins), s>>>(descs, in, out, n, queue, slots, qmask, wait_limit_ns, P)
   KF_ASSOC_SWITCH(P, KF_X);
 #undef KF_X
   return cudaGetLastError();

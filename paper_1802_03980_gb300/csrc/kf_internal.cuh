@@ -329,9 +329,10 @@ cudaError_t launch_integral_normals(const DescList& list, int max_w, int max_h, 
 cudaError_t launch_model_prep(const PairDesc& desc, PairDesc* d_desc, const float* V, const float* N, int w,
                               int h, int precision, cudaStream_t s);
 // the shared memory that the variant's kernels may take (before any query or
-// launch of them in a context)
-void icp_attributes(const KParams& P);
-void team_attributes(const KParams& P);
+// launch of them in a context): the attribute belongs to the kernel, not to a
+// tracker, so it is always that of the most bins
+cudaError_t icp_attributes(const KParams& P);
+cudaError_t team_attributes(const KParams& P);
 // grid sizes (one wave) of the per-stage and the scheduled ICP kernels
 void icp_grids(const KParams& P, int* g_assoc, int* g_reduce, int* g_sched);
 cudaError_t launch_icp_init(const PairDesc* const* descs, const PairInput* in, int n, int* list,

@@ -603,12 +603,14 @@ __global__ void __launch_bounds__(kTeamBlock, 1) k_icp_team(const __grid_constan
 
 }  // namespace
 
-void team_attributes(const KParams& P) {
-#define KF_X(T, A)                                                                     \
-  cudaFuncSetAttribute(k_icp_team<T, A>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                       P.bins * (int)sizeof(unsigned))
+cudaError_t team_attributes(const KParams& P) {
+  cudaError_t e = cudaSuccess;
+#define KF_X(T, A)                                                                         \
+  e = cudaFuncSetAttribute(k_icp_team<T, A>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                           kMaxBins * (int)sizeof(unsigned))
   KF_ASSOC_SWITCH(P, KF_X);
 #undef KF_X
+  return e;
 }
 
 int team_blocks(const KParams& P) {
