@@ -1174,8 +1174,7 @@ namespace kf {
 namespace {
 
 constexpr int kNoAllocMaxItems = 1024;  // 1024 items x 4096 px = 4,194,304 frame pixels
-constexpr size_t kNoAllocHeader = 512;  // arrival counters
-constexpr int kNoAllocCounters = 64;    // taken in turn by the calls
+constexpr size_t kNoAllocHeader = 512;  // the arrivals' word
 constexpr int kNoAllocStride = 32;     // floats per block partial (29 used)
 constexpr size_t kNoAllocBytes = kNoAllocHeader + sizeof(float) * kNoAllocStride * kNoAllocMaxItems;
 constexpr int kNoAllocMaxDevices = 64;
@@ -1194,15 +1193,19 @@ struct NoAllocArgs {
   double Tm[12];              // model pose 3x4
   KParams P;                  // d_max32, scale32, bins, tiny_bins used
   int klo, khi;
-  int counter;                // arrival counter of this call, of kNoAllocCounters
+  unsigned long long first;   // the arrivals' word before this call's first arrival
   double* out;                // 29 sums (device)
 };
 
 // One block per item of 4096 frame pixels; the last block to arrive adds the
-// items (ItemSum). A thread takes its pixels kNoAllocFly at a time, every load
-// of a batch before its first use, then adds the rows in pixel order: what
-// bounds it is the two round trips of a batch (vertices, then model pixels),
-// which a pixel-by-pixel loop pays 16 times over. kShort: a model up to 2^22
+// items (ItemSum). The arrivals' word holds the number of the call in its upper
+// half, so a call starts from zero whatever an earlier one left there: each block
+// raises the word to the call's first value (a store that nobody waits for)
+// before it counts itself. A captured call has the same number in every replay; a
+// node of its own zeroes the word there. A thread takes its pixels kNoAllocFly
+// at a time, every load of a batch before its first use, then adds the rows in
+// pixel order: what bounds it is the two round trips of a batch (vertices, then
+// model pixels), which a pixel-by-pixel loop pays 16 times over. kShort: a model up to 2^22
 // pixels wide and high and no tiny bins (see project, bin_of).
 // Measured on GB300, 640x480: 28.4 us with a set-up launch, pixel by pixel and
 // a float64 chain over the items; 13.3 us now (calls in a row, the host's
@@ -1215,7 +1218,8 @@ __global__ void __launch_bounds__(kBlock) k_noalloc_reduce(unsigned char* scratc
   __shared__ float s_red[kBlock / 32][kSums];
   __shared__ ItemSumWord s_part_raw[kBlock / 32][kSums];
   __shared__ int s_last;
-  unsigned* counter = reinterpret_cast<unsigned*>(scratch) + a.counter;
+  unsigned long long* arrivals = reinterpret_cast<unsigned long long*>(scratch);
+  if (threadIdx.x == 0) atomicMax(arrivals, a.first);
   float* partials = reinterpret_cast<float*>(scratch + kNoAllocHeader);
   const int npx = a.fw * a.fh;
   const int begin = blockIdx.x * kChunk;
@@ -1312,7 +1316,7 @@ __global__ void __launch_bounds__(kBlock) k_noalloc_reduce(unsigned char* scratc
     __threadfence();
   }
   __syncthreads();
-  if (threadIdx.x == 0) s_last = (atomicAdd(counter, 1u) == (unsigned)(nitems - 1));
+  if (threadIdx.x == 0) s_last = atomicAdd(arrivals, 1ull) == a.first + (unsigned)(nitems - 1);
   __syncthreads();
   if (!s_last) return;
   __threadfence();
@@ -1326,12 +1330,7 @@ __global__ void __launch_bounds__(kBlock) k_noalloc_reduce(unsigned char* scratc
   }
   __syncthreads();
   if (threadIdx.x < kSums) a.out[threadIdx.x] = total_of(part, threadIdx.x, shift);
-  // this call's counter, and the one a call half the ring later will use
-  // (should overlapping calls have left it wrong)
-  if (threadIdx.x == 0) {
-    *counter = 0u;
-    reinterpret_cast<unsigned*>(scratch)[(a.counter + kNoAllocCounters / 2) % kNoAllocCounters] = 0u;
-  }
+  if (threadIdx.x == 0) *arrivals = 0ull;
 }
 
 std::mutex g_noalloc_mutex;
@@ -1396,8 +1395,15 @@ extern "C" kf_status kf_reduce_noalloc(const float* frame_vertex, int width, int
   a.out = sums;
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   const int nitems = (int)((npx + kChunk - 1) / kChunk);
-  static std::atomic<unsigned> next_call{0};
-  a.counter = (int)(next_call.fetch_add(1) % kNoAllocCounters);
+  static std::atomic<unsigned> next_call{1};
+  a.first = (unsigned long long)next_call.fetch_add(1) << 32;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(s, &capture);
+  if (e == cudaSuccess && capture == cudaStreamCaptureStatusActive) e = cudaMemsetAsync(scratch, 0, sizeof(a.first), s);
+  if (e != cudaSuccess) {
+    (void)cudaGetLastError();
+    return KF_ERR_CUDA;
+  }
   a.P.tiny_bins = tiny_bins(a.P.d_max32, a.P.scale32);
   const bool brief = !a.P.tiny_bins && a.mw <= (1 << 22) && a.mh <= (1 << 22);
   auto kernel = brief ? k_noalloc_reduce<true> : k_noalloc_reduce<false>;
