@@ -369,7 +369,8 @@ const char* kf_volume_last_error(const kf_volume* v);
 kf_status kf_volume_reset(kf_volume* v);
 /* Fuse a raw depth frame (W x H float32 metres, host memory copied before
  * return, or device memory read by the queued kernel) seen from the
- * camera->world pose (row-major 4x4 FP64) with intrinsics K. */
+ * camera->world pose (row-major 4x4 FP64) with intrinsics K. A device frame's
+ * call only queues work: it can be captured. */
 kf_status kf_volume_integrate(kf_volume* v, const float* depth, const kf_intrinsics* K,
                               const double pose[16], int is_device_ptr);
 /* Vertex and normal maps (K->width x K->height x 3 float32 each) of the field

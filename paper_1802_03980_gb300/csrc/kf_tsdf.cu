@@ -118,6 +118,10 @@ __device__ __forceinline__ int pixel_of(float f, float p, float pz, float y, flo
 // than that depth plus mu is not updated.
 constexpr int kBrick = 8;
 constexpr int kDepthTile = 16;
+// Tiles that a volume holds: frames up to 4096 x 4096 (larger ones are not tested
+// against the depth). Allocated with it, since an integration allocates nothing
+// for a device frame: it can be captured.
+constexpr int kMaxTiles = 65536;
 struct Frustum {
   float n[4][3];  // unit normals of the side planes (camera frame), inside: n . p >= 0
   float fx, fy, cx, cy;   // for the tiles (fx, fy > 0)
@@ -494,14 +498,14 @@ struct kf_volume {
   bool own_stream = false;
   float2* FW = nullptr;     // field and weight of each voxel
   NearMap near = {};
-  float* tiles = nullptr;   // largest depth per tile of the frame being integrated (grown on demand)
-  size_t tiles_cap = 0;
+  float* tiles = nullptr;   // [kMaxTiles] largest depth per tile of the frame being integrated
   float* depth = nullptr;   // staging for host frames (grown on demand)
   size_t depth_cap = 0;
   float* maps = nullptr;    // staging for host outputs (grown on demand)
   size_t maps_cap = 0;
   int nb = 0;               // bricks per edge
-  int* bricks = nullptr;    // kept bricks of the current integration
+  int* bricks = nullptr;    // kept bricks of the current integration (also what kf_volume_read takes apart)
+  size_t bricks_cap = 0;    // ints
   unsigned* brick_count = nullptr;
   int sms = 1;
   std::string err;
@@ -614,7 +618,9 @@ kf_status kf_volume_create(const kf_volume_params* p, void* cuda_stream, kf_volu
   const size_t nb3 = (size_t)v->nb * v->nb * v->nb, ns3 = (size_t)v->near.ns * v->near.ns * v->near.ns;
   if (e == cudaSuccess) e = cudaMalloc(&v->near.brick, nb3 + ns3);
   v->near.super = v->near.brick + nb3;
-  if (e == cudaSuccess) e = cudaMalloc(&v->bricks, (size_t)v->nb * v->nb * v->nb * sizeof(int));
+  v->bricks_cap = std::max(nb3, (size_t)1 << 16);
+  if (e == cudaSuccess) e = cudaMalloc(&v->bricks, v->bricks_cap * sizeof(int));
+  if (e == cudaSuccess) e = cudaMalloc(&v->tiles, kMaxTiles * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&v->brick_count, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&v->sms, cudaDevAttrMultiProcessorCount, v->device);
   if (e != cudaSuccess) {
@@ -695,11 +701,9 @@ kf_status kf_volume_integrate(kf_volume* v, const float* depth, const kf_intrins
   const int nb = v->nb;
   const int nbricks = nb * nb * nb;
   const int tw = (K->width + kDepthTile - 1) / kDepthTile, th = (K->height + kDepthTile - 1) / kDepthTile;
-  // tile sizes and the projection in float32 pixels: images of sane size only
-  const bool tiled = K->fx > 0.0 && K->fy > 0.0 && K->width <= 65536 && K->height <= 65536;
+  // the projection in float32 pixels: images of sane size only
+  const bool tiled = K->fx > 0.0 && K->fy > 0.0 && K->width <= 65536 && K->height <= 65536 && (long long)tw * th <= kMaxTiles;
   if (tiled) {
-    kf_status st = grow(v, &v->tiles, &v->tiles_cap, sizeof(float) * tw * th);
-    if (st != KF_OK) return st;
     fr.fx = (float)K->fx;
     fr.fy = (float)K->fy;
     fr.cx = (float)K->cx;
@@ -778,20 +782,17 @@ kf_status kf_volume_read(kf_volume* v, float* F, float* W) {
   if (!v) return KF_ERR_INVALID_ARG;
   const size_t n = (size_t)v->g.res * v->g.res * v->g.res;
   KV_CK(v, cudaStreamSynchronize(v->stream));
-  const size_t most = std::min(n, (size_t)1 << 24);  // voxels taken apart at a time
-  float* part = nullptr;
-  KV_CK(v, cudaMalloc(&part, 2 * most * sizeof(float)));
-  cudaError_t e = cudaSuccess;
-  for (size_t at = 0; at < n && e == cudaSuccess; at += most) {
+  // a part of the volume at a time, taken apart in the brick list (the stream is idle)
+  const size_t most = v->bricks_cap / 2;
+  float* part = reinterpret_cast<float*>(v->bricks);
+  for (size_t at = 0; at < n; at += most) {
     const size_t m = std::min(most, n - at);
     k_split<<<1216, 256, 0, v->stream>>>(v->FW + at, m, part, part + most);
-    e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(v->stream);
-    if (e == cudaSuccess && F) e = cudaMemcpy(F + at, part, m * sizeof(float), cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess && W) e = cudaMemcpy(W + at, part + most, m * sizeof(float), cudaMemcpyDeviceToHost);
+    KV_CK(v, cudaGetLastError());
+    KV_CK(v, cudaStreamSynchronize(v->stream));
+    if (F) KV_CK(v, cudaMemcpy(F + at, part, m * sizeof(float), cudaMemcpyDeviceToHost));
+    if (W) KV_CK(v, cudaMemcpy(W + at, part + most, m * sizeof(float), cudaMemcpyDeviceToHost));
   }
-  cudaFree(part);
-  KV_CK(v, e);
   return KF_OK;
 }
 
