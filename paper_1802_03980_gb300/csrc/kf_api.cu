@@ -370,8 +370,9 @@ bool plan_teams(kf_tracker* const* trk, Plan* pl) {
   return pl->grid <= t0->team_blocks;
 }
 
-// Queues the team launch of a plan whose inputs are in h_in.
-kf_status launch_teams(kf_tracker* const* trk, Plan* pl, cudaStream_t s) {
+// Queues the team launch of a plan whose inputs are in h_in. refused: the device
+// would not hold all its blocks at once (a context with a part of the SMs, say).
+kf_status launch_teams(kf_tracker* const* trk, Plan* pl, cudaStream_t s, bool* refused) {
   kf_tracker* t0 = trk[0];
   for (int k = 0; k < pl->n; ++k) {
     kf_tracker* t = trk[pl->order[k]];
@@ -391,7 +392,10 @@ kf_status launch_teams(kf_tracker* const* trk, Plan* pl, cudaStream_t s) {
     KF_CK(t0, cudaEventRecord(pl->ev[0], s));
     KF_CK(t0, cudaEventRecord(pl->ev[1], s));
   }
-  KF_CK(t0, launch_icp_team(pl->args, pl->grid, t0->kp, s));
+  const cudaError_t e = launch_icp_team(pl->args, pl->grid, t0->kp, s);
+  *refused = e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported;
+  if (*refused) (void)cudaGetLastError();
+  KF_CK(t0, e);
   if (pl->profiled) KF_CK(t0, cudaEventRecord(pl->ev[2], s));
   return KF_OK;
 }
@@ -993,19 +997,31 @@ kf_status kf_align_batch(kf_tracker* const* trk, int n, const double* prior_R,
     }
     Plan* pl = *slot;
     cudaStream_t s = t0->stream;
-    for (int k = 0; k < n; ++k) {  // device pair k: the caller's pair i
-      const int i = pl->order[k];
-      PairInput& in = pl->h_in[k];
-      memset(&in, 0, sizeof(in));
-      if (prior_R) memcpy(in.prior_R, prior_R + 9 * i, sizeof(double) * 9);
-      memcpy(in.init, init_pose + 16 * i, sizeof(double) * 16);
-      in.lambda = lambda[i] < 0 ? t0->p.lambda_c : lambda[i];
-      in.has_prior = prior_R ? 1 : 0;
-    }
+    auto inputs = [&] {
+      for (int k = 0; k < n; ++k) {  // device pair k: the caller's pair i
+        const int i = pl->order[k];
+        PairInput& in = pl->h_in[k];
+        memset(&in, 0, sizeof(in));
+        if (prior_R) memcpy(in.prior_R, prior_R + 9 * i, sizeof(double) * 9);
+        memcpy(in.init, init_pose + 16 * i, sizeof(double) * 16);
+        in.lambda = lambda[i] < 0 ? t0->p.lambda_c : lambda[i];
+        in.has_prior = prior_R ? 1 : 0;
+      }
+    };
+    inputs();
+    bool refused = false;
     if (pl->team) {
       // inputs in the launch's parameters, outputs written to pinned host memory
-      kf_status st = launch_teams(trk, pl, s);
+      kf_status st = launch_teams(trk, pl, s, &refused);
+      if (refused) {  // the queue's launch runs with any number of blocks
+        t0->team_blocks = 0;
+        st = build_plan(trk, n, slot);
+        pl = *slot;
+      }
       if (st != KF_OK) return st;
+      if (refused) inputs();
+    }
+    if (pl->team) {
       KF_CK(t0, cudaStreamSynchronize(s));
       for (int k = 0; k < n; ++k) {
         const int st = pl->h_out[k].res.status;

@@ -54,6 +54,10 @@ namespace {
 constexpr int kTeamWarps = 4;            // item warps of a half item
 static_assert(kTeamWarps * kTeamPlaces == level_chunk(0) / 2, "record places of a half item");
 constexpr int kTeamBlock = 2 * 32 * kTeamWarps;  // two warps (parts) for each
+// blocks per SM that a launch may count on; 0: what the device says
+#ifndef KF_TEAM_PER_SM
+#define KF_TEAM_PER_SM 0
+#endif
 constexpr int kPollCheck = 64;  // polls between two looks at the clock
 // pause between two polls of a worker without half items at its level
 #ifndef KF_TEAM_IDLE_NS
@@ -621,7 +625,7 @@ int team_blocks(const KParams& P) {
 #define KF_X(T, A) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_icp_team<T, A>, kTeamBlock, sm)
   KF_ASSOC_SWITCH(P, KF_X);
 #undef KF_X
-  return sms * per;
+  return sms * (KF_TEAM_PER_SM > 0 ? KF_TEAM_PER_SM : per);
 }
 
 cudaError_t launch_icp_team(const TeamArgs& args, int grid, const KParams& P, cudaStream_t s) {
