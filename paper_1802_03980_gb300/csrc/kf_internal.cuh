@@ -153,9 +153,17 @@ __host__ __device__ constexpr int team_hist_words(int bins) { return team_hist_n
 constexpr unsigned kTeamHists = 16;   // rotating histograms, a power of two
 constexpr unsigned kTeamAcquire = 8;  // iterations between two acquires, a power of two
 static_assert(kTeamHists >= kTeamAcquire + 1 + 2, "a clear comes before the messages of two iterations on");
+// Half items of a worker at most: beyond, the queue's blocks, which share all
+// items of all pairs, come near the team's whole slots. Measured on GB300, set
+// frame and align of a batch, team against queue, us: one slot a worker 162 / 302
+// (one pair 640x480), two 183 / 338 (700x525), 178 / 321 (800x600) and 179 / 314
+// (two 640x480), four 272 / 430 (1280x960), seven 417 / 580 (1920x1080) and 356 /
+// 434 (six 640x480), eight 391 / 456 (seven).
 constexpr int kTeamSlots = 8;
 constexpr int kTeamPlaces = level_chunk(0) / kBlockWarps;  // record places of an item warp, at any level
 constexpr int kTeamMaxItems = 1024;  // items of the largest frame
+// pairs whose inputs go with the launch; 16 pairs 320x240: 308 us team, 424 queue,
+// 160x120: 256 and 424
 constexpr int kTeamMaxPairs = 16;
 
 struct DescList {
