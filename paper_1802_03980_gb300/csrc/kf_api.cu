@@ -375,20 +375,27 @@ bool plan_teams(kf_tracker* const* trk, Plan* pl) {
   return pl->grid <= t0->team_blocks;
 }
 
+// The tag of the tracker's next team launch. A tag repeats after 2^20 launches:
+// start again from zeroed buffers then, and after a launch that ended before its
+// last clear.
+kf_status team_tag(kf_tracker* t, cudaStream_t s, unsigned* tag) {
+  if (t->team_dirty || (t->team_epoch + 1) * (unsigned long long)kTeamTags >= (1ull << 32)) {
+    KF_CK(t, cudaMemsetAsync(t->d_team, 0, t->team_bytes, s));
+    t->team_epoch = 0;
+  }
+  t->team_dirty = true;  // until the outputs say otherwise
+  *tag = ++t->team_epoch * kTeamTags;
+  return KF_OK;
+}
+
 // Queues the team launch of a plan whose inputs are in h_in. refused: the device
 // would not hold all its blocks at once (a context with a part of the SMs, say).
 kf_status launch_teams(kf_tracker* const* trk, Plan* pl, cudaStream_t s, bool* refused) {
   kf_tracker* t0 = trk[0];
   for (int k = 0; k < pl->n; ++k) {
     kf_tracker* t = trk[pl->order[k]];
-    // a tag repeats after 2^20 launches: start again from zeroed buffers then,
-    // and after a launch that ended before its last clear
-    if (t->team_dirty || (t->team_epoch + 1) * (unsigned long long)kTeamTags >= (1ull << 32)) {
-      KF_CK(t0, cudaMemsetAsync(t->d_team, 0, t->team_bytes, s));
-      t->team_epoch = 0;
-    }
-    t->team_dirty = true;  // until the outputs say otherwise
-    pl->args.pair[k].tag = ++t->team_epoch * kTeamTags;
+    const kf_status st = team_tag(t, s, &pl->args.pair[k].tag);
+    if (st != KF_OK) return st;
     pl->args.pair[k].out = pl->h_out + k;
     pl->args.in[k] = pl->h_in[k];
     pl->h_out[k].res.status = KF_ERR_TIMEOUT;
@@ -1257,10 +1264,13 @@ kf_status kf_debug_wait_timeout(kf_tracker* t, double wait_ms) {
       out->res.status = KF_ERR_TIMEOUT;
       args.pair[0].d = t->d_desc;
       args.pair[0].out = out;
-      args.pair[0].tag = ++t->team_epoch * kTeamTags;
+      const kf_status ts = team_tag(t, s, &args.pair[0].tag);
+      if (ts != KF_OK) {
+        cudaFreeHost(out);
+        return ts;
+      }
       args.n = 1;
       args.limit_ns = (unsigned long long)(ms * 1e6);
-      t->team_dirty = true;
       e = launch_icp_team(args, 1, t->kp, s);
       if (e == cudaSuccess) e = cudaStreamSynchronize(s);
       const int st = out->res.status;
