@@ -510,7 +510,7 @@ __device__ void reduce_items(const PairDesc* d, const LevelMaps& L, int first, i
 // solve's next level (-1: finished or stopped).
 __device__ __noinline__ int combine_and_solve(const PairDesc* d, PairState* st, int count,
                                                int level, const KParams& P, int mode,
-                                               ItemSum (*s_part)[kSums], double* s_sums) {
+                                               SubSums& s_part, double* s_sums) {
   __shared__ int s_hit;
   PairPre pre;
   if (threadIdx.x == 0) {
@@ -542,26 +542,28 @@ __device__ __noinline__ int combine_and_solve(const PairDesc* d, PairState* st, 
       for (int i = 0; i < h; ++i) v[i] = __fadd_rn(v[i], v[i + h]);
     return v[0];
   };
-  const int shift = sum_shift(count);
-  ItemSum t;
+  static_assert(kItemFold % 4 == 0, "folds where the other launches have them");
+  FoldedSum t;
   if (k < kSums) {
     int l = sub;
     for (; l + 24 < count; l += 32) {
       const float e0 = item_value(l), e1 = item_value(l + 8), e2 = item_value(l + 16),
                   e3 = item_value(l + 24);
-      t.add(e0, shift);
-      t.add(e1, shift);
-      t.add(e2, shift);
-      t.add(e3, shift);
+      t.room(4);
+      t.s.add(e0);
+      t.s.add(e1);
+      t.s.add(e2);
+      t.s.add(e3);
     }
-    for (; l < count; l += 8) t.add(item_value(l), shift);
-    s_part[sub][k] = t;
+    for (; l < count; l += 8) {
+      t.room(1);
+      t.s.add(item_value(l));
+    }
+    s_part.put(sub, k, t, count);
   }
   for (int b = threadIdx.x; b < P.bins; b += kBlock) d->hist[b] = 0u;
   __syncthreads();
-  if (threadIdx.x < kSums) {
-    s_sums[threadIdx.x] = total_of(s_part, threadIdx.x, shift);
-  }
+  if (threadIdx.x < kSums) s_sums[threadIdx.x] = s_part.total(threadIdx.x, count);
   __syncthreads();
   int next = -1;
   if (threadIdx.x < 32) {
@@ -660,8 +662,7 @@ __global__ void __launch_bounds__(kBlock, KF_REDUCE_MINB) k_reduce_solve(const P
   __shared__ __align__(16) float sxf[24];  // 16-byte vector loads (load_xf)
   __shared__ int s_active, s_klo, s_khi, s_hit, s_last;
   __shared__ double s_sums[kSums];
-  __shared__ ItemSumWord s_part_raw[8][kSums];
-  ItemSum (*s_part)[kSums] = reinterpret_cast<ItemSum (*)[kSums]>(s_part_raw);
+  __shared__ SubSums s_part;
   const int n_items = __ldcg(list);
   const int M = (n_items + gridDim.x - 1) / gridDim.x;
   int f = blockIdx.x * M;
@@ -936,8 +937,7 @@ __global__ void __launch_bounds__(kBlock, KF_SCHED_MINB) k_icp_sched(const PairD
   __shared__ unsigned long long s_word;
   __shared__ int s_last, s_flag, s_a, s_b, s_hit;
   __shared__ double s_sums[kSums];
-  __shared__ ItemSumWord s_part_raw[8][kSums];
-  ItemSum (*s_part)[kSums] = reinterpret_cast<ItemSum (*)[kSums]>(s_part_raw);
+  __shared__ SubSums s_part;
   __shared__ double s_seed[12];
   // seed: every block that starts takes unseeded pairs until none is left
   for (;;) {
@@ -1216,7 +1216,7 @@ __global__ void __launch_bounds__(kBlock) k_noalloc_reduce(unsigned char* scratc
                                                            const __grid_constant__ NoAllocArgs a, int nitems) {
   __shared__ __align__(16) float sxf[24];  // 16-byte vector loads (load_xf)
   __shared__ float s_red[kBlock / 32][kSums];
-  __shared__ ItemSumWord s_part_raw[kBlock / 32][kSums];
+  __shared__ SubSums s_part;
   __shared__ int s_last;
   unsigned long long* arrivals = reinterpret_cast<unsigned long long*>(scratch);
   if (threadIdx.x == 0) atomicMax(arrivals, a.first);
@@ -1320,16 +1320,18 @@ __global__ void __launch_bounds__(kBlock) k_noalloc_reduce(unsigned char* scratc
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  ItemSum (*part)[kSums] = reinterpret_cast<ItemSum (*)[kSums]>(s_part_raw);
-  const int shift = sum_shift(nitems);
   if (lane < kSums) {
-    ItemSum t;
+    FoldedSum t;
+    for (int l0 = warp; l0 < nitems; l0 += kItemFold * (kBlock / 32)) {
+      const int l1 = min(nitems, l0 + kItemFold * (kBlock / 32));
+      t.room(kItemFold);
 #pragma unroll 8
-    for (int l = warp; l < nitems; l += kBlock / 32) t.add(__ldcg(partials + l * kNoAllocStride + lane), shift);
-    part[warp][lane] = t;
+      for (int l = l0; l < l1; l += kBlock / 32) t.s.add(__ldcg(partials + l * kNoAllocStride + lane));
+    }
+    s_part.put(warp, lane, t, nitems);
   }
   __syncthreads();
-  if (threadIdx.x < kSums) a.out[threadIdx.x] = total_of(part, threadIdx.x, shift);
+  if (threadIdx.x < kSums) a.out[threadIdx.x] = s_part.total(threadIdx.x, nitems);
   if (threadIdx.x == 0) *arrivals = 0ull;
 }
 

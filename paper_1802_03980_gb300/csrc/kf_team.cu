@@ -169,7 +169,7 @@ struct TeamShared {
   float row[2][kTeamWarps][32];
   int count[kTeamSlots][kTeamWarps][2];  // records of each part
   double T[12];
-  ItemSumWord part[kBlockWarps][kSums];
+  SubSums part;
   double sums[kSums + 3];
   int level, w0, w1;
   unsigned it;
@@ -492,15 +492,14 @@ __device__ void team_lead(const PairDesc* d, const TeamPair& tp, const PairInput
       if (warp == 0) next = next_step(pre, level, P);
       // per sum (lane) the items' values: sub-sums over items sub, sub + 8, ...
       // (combine_and_solve's order)
-      ItemSum (*part)[kSums] = reinterpret_cast<ItemSum (*)[kSums]>(sh.part);
-      const int shift = sum_shift(count);
       const unsigned long long want = tp.tag + it;
       Wait wait;
       bool ok = true;
       // a warp reads its sub-sum's packets together: one round trip covers 80
       // items (a 640x480 frame has 75)
       constexpr int kLeadWarps = kTeamBlock / 32, kSubs = kBlockWarps / kLeadWarps, kFly = 10;
-      ItemSum sub[kSubs];
+      static_assert(kItemFold % kFly == 0, "folds where the other launches have them");
+      FoldedSum sub[kSubs];
       for (int l0 = warp; l0 < count && ok; l0 += kFly * kBlockWarps) {
         unsigned long long a[kSubs][kFly], b[kSubs][kFly];
         for (;;) {
@@ -527,19 +526,21 @@ __device__ void team_lead(const PairDesc* d, const TeamPair& tp, const PairInput
           }
         }
 #pragma unroll
-        for (int j = 0; j < kSubs; ++j)
+        for (int j = 0; j < kSubs; ++j) {
+          sub[j].room(kFly);
 #pragma unroll
           for (int i = 0; i < kFly; ++i)
             if (l0 + j * kLeadWarps + i * kBlockWarps < count)
-              sub[j].add(__fadd_rn(__uint_as_float((unsigned)a[j][i]), __uint_as_float((unsigned)b[j][i])), shift);
+              sub[j].s.add(__fadd_rn(__uint_as_float((unsigned)a[j][i]), __uint_as_float((unsigned)b[j][i])));
+        }
       }
       if (lane < kSums)
-        for (int j = 0; j < kSubs; ++j) part[warp + j * kLeadWarps][lane] = sub[j];
+        for (int j = 0; j < kSubs; ++j) sh.part.put(warp + j * kLeadWarps, lane, sub[j], count);
       if (!ok) sh.abort = 1;
       __syncthreads();
       if (sh.abort) return;
       if (warp == 0) {
-        if (lane < kSums) sh.sums[lane] = total_of(part, lane, shift);
+        if (lane < kSums) sh.sums[lane] = sh.part.total(lane, count);
         __syncwarp();
         double Tc[3];
 #pragma unroll
