@@ -1,11 +1,15 @@
 """Autotuner of the ICP kernels' compile-time shapes.
 
 The scheduled ICP kernel has shapes that only a measurement can choose: how
-many frame pixels a thread takes per batch (KF_ASSOC_U), how many blocks an
-SM holds (KF_SCHED_MINB, which caps the registers), the band-edge windows of
-the association pass (KF_WIN_*), the L2 hints (KF_PREFETCH), how long the
-queue's tasks run (KF_RUNS_PER_BLOCK, KF_MAX_RUN) and from how many running
-pairs a pair's median block also runs its reduction pass (KF_FUSE_GRID_DIV).
+many frame pixels a thread takes per batch of the association's ring and how
+many batches ahead their model records are sent for (KF_RING_U, KF_RING_AHEAD),
+how many blocks an SM holds (KF_SCHED_MINB, which caps the registers), the
+band-edge windows of the association pass (KF_WIN_*), how long the queue's tasks
+run (KF_RUNS_PER_BLOCK, KF_MAX_RUN) and from how many running pairs a pair's
+median block also runs its reduction pass (KF_FUSE_GRID_DIV). The gated and
+shooting variants gather through registers instead of the ring: KF_ASSOC_U and
+KF_PREFETCH are theirs (and the per-iteration launches'). The batch that is timed
+takes the queue's launch, however few pairs are asked for.
 The tuner:
 
 1. builds one library per candidate (the tuning macros as -D defines), in
@@ -44,8 +48,19 @@ TUNED = os.path.join(HERE, "tuned.json")
 GRID = {
     "KF_RUNS_PER_BLOCK": [2, 3],
     "KF_FUSE_GRID_DIV": [4, 0],
-    "KF_PREFETCH": [1, 0],
+    "KF_RING_U": [2, 1],
+    "KF_RING_AHEAD": [1, 2],
 }
+
+# the fewest pairs that always take the queue's launch: one more than a team
+# launch takes
+QUEUE_PAIRS = 17
+
+
+def queue_batch(pairs: int) -> list[int]:
+    """The pair of each tracker that is timed: every pair once, then again from
+    the first on until the batch is too large for a team launch."""
+    return [i % pairs for i in range(max(pairs, QUEUE_PAIRS))]
 
 
 def candidates(grid: dict) -> list[dict]:
@@ -87,25 +102,27 @@ def _worker(data: str, steps: int, warmup: int, precision: int) -> dict:
     p = kf.kf_default_params()
     p.precision = precision
     stream = torch.cuda.Stream()
-    trk = [kf.kf_track_create(p, K[0], K[1], stream.cuda_stream) for _ in range(n)]
+    of = queue_batch(n)
+    trk = [kf.kf_track_create(p, K[0], K[1], stream.cuda_stream) for _ in of]
     try:
         depth = np.ascontiguousarray(z["depth"], np.float32)
         mv = np.ascontiguousarray(z["mv"], np.float32)
         mn = np.ascontiguousarray(z["mn"], np.float32)
-        for i, t in enumerate(trk):  # the arrays above stay alive across the calls
+        prior_R, init_pose, lam = z["prior_R"][of], z["init_pose"][of], z["lam"][of]
+        for i, t in zip(of, trk):  # the arrays above stay alive across the calls
             kf.kf_set_frame(t, depth[i].ctypes.data, K, False)
             kf.kf_set_model(t, mv[i].ctypes.data, mn[i].ctypes.data, z["model_pose"][i], K, False)
         for _ in range(warmup):
-            kf.kf_align_batch(trk, z["prior_R"], z["init_pose"], z["lam"])
+            kf.kf_align_batch(trk, prior_R, init_pose, lam)
         kf.kf_profile_enable(trk[0], 1)
         for _ in range(steps):
-            st, poses, res = kf.kf_align_batch(trk, z["prior_R"], z["init_pose"], z["lam"])
+            st, poses, res = kf.kf_align_batch(trk, prior_R, init_pose, lam)
         prof = kf.kf_profile_read(trk[0])
         kf.kf_profile_enable(trk[0], 0)
-        return {"status": int(st), "poses": poses.tolist(),
+        return {"status": int(st), "poses": poses[:n].tolist(),
                 "launch_ms": prof.sched_ms / max(1, prof.sched_launches),
                 "align_ms": prof.align_ms / max(1, prof.graph_launches),
-                "iters": [list(r.iters) for r in res]}
+                "iters": [list(r.iters) for r in res[:n]]}
     finally:
         for t in trk:
             kf.kf_track_destroy(t)
