@@ -5,8 +5,8 @@ One step = the whole hot path over one batch of synthetic Kinect-sized frame
 pairs already resident in HBM: bilateral filter, depth pyramid, vertex and
 normal maps (kf_set_frame_batch), then the coarse-to-fine regularised ICP
 with the distance histogram, median filter and convergence control
-(kf_align_batch, one CUDA graph). The value is alignments per second over
-all ranks; e2e repeats the measurement with the depth frames copied from
+(kf_align_batch, one persistent launch). The value is alignments per second
+over all ranks; e2e repeats the measurement with the depth frames copied from
 pinned host memory and the poses read back every step, pipelined as a
 serving loop would run it (two tracker sets: the copy engine uploads the
 next batch while the current one aligns), with the one-batch-at-a-time
@@ -39,13 +39,15 @@ UNIT = "alignments/s"
 W, H = 640, 480
 CAPS = (10, 5, 4)
 LAM = 1e3
-# ncu DRAM bytes (read + write) of the dominant kernel per pixel-iteration,
-# by (kernel, precision), from the captures summarised in profiles/ for the
-# kernel as it stands: one launch over 64 pairs of 640x480 each (FP32:
-# 3.477 + 0.189 GB over 82,310,400 pixel-iterations; FP16: 1.801 + 0.171 GB
-# over 83,980,800). Larger batches are scaled by the pixel-iterations their
-# launch processes (the traffic per pixel-iteration does not depend on how
-# many independent pairs share the launch).
+# ncu DRAM bytes (read + write) of the ICP launch per pixel-iteration, by
+# precision, from profiles/k_icp_sched_k_frontend_current.md: one launch over 64
+# pairs of 640x480. Larger batches are scaled by the pixel-iterations their launch
+# processes (the traffic per pixel-iteration does not depend on how many
+# independent pairs share the launch).
+NCU_DRAM_PER_PX_ITER = {"fp32": (3688177152 + 179900160) / 82310400,
+                        "fp16": (1942506752 + 168679680) / 83980800}
+# the same of the launch before its maps became records and its gathers
+# asynchronous copies; no figure of the line uses it
 NCU_TRAFFIC_PER_PX_ITER = {("k_icp_sched", "fp32"): (3477426688 + 188985088) / 82310400,
                            ("k_icp_sched", "fp16"): (1800692224 + 170857472) / 83980800}
 
@@ -478,7 +480,7 @@ def precision_form(kf, torch, pairs, stream, steps, oracle, main=None):
     trk = [kf.kf_track_create(p, mw, mh, stream.cuda_stream) for _ in range(ns)]
     try:
         _models_to_device(kf, torch, trk, pairs[:ns], stream)
-        for i in range(ns):  # builds each tracker's single-pair graph
+        for i in range(ns):  # builds each tracker's single-pair plan
             kf.kf_set_frame(trk[i], dptrs[i], Ks[i], True)
             kf.kf_align(trk[i], priors[i], inits[i], lams[i])
         torch.cuda.synchronize()
@@ -707,7 +709,7 @@ def gb300_arm(args):
     achieved = bytes_per_launch / (kms / max(1, klaunch) / 1000.0) / 1e9 if kms > 0 else 0.0
     # DRAM bytes of one launch of this kernel on this workload, from ncu
     # (dram__bytes_read.sum + dram__bytes_write.sum); null when not captured
-    per_px = NCU_TRAFFIC_PER_PX_ITER.get((dom, args.precision)) if wl == "kinect640" else None
+    per_px = NCU_DRAM_PER_PX_ITER[args.precision] if wl == "kinect640" and dom == "k_icp_sched" else None
     traffic = per_px * (px_iters * args.steps / max(1, klaunch)) if per_px else None
     corr = prof.pixel_iters / (prof.align_ms / 1000.0) / 1e6 if prof.align_ms > 0 else None
     # kernels of ours per step: the front end, then the scheduled launch, or
@@ -765,7 +767,7 @@ def gb300_arm(args):
                                   "page-locked buffer (one copy per batch)",
                 "one_batch_at_a_time": e2e_serial_value,
                 "one_batch_at_a_time_form": "one tracker set; set-frame pulls the page-locked frames "
-                                            "with one gather kernel, align returns the poses",
+                                            "(the first by a gather kernel, the rest by the front end), align returns the poses",
                 "model_maps": "resident: set once before the timed region, not uploaded per step",
                 "with_model_upload": {"value": e2e_model_value, "steps": nm,
                                       "h2d_bytes_per_step": h2d + h2d_model,
