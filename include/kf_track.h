@@ -195,8 +195,10 @@ void kf_track_destroy(kf_tracker* t);
 /* Where kf_set_frame / kf_set_frame_batch find the depth (is_device_ptr). */
 #define KF_FRAME_HOST 0              /* host memory: pageable frames are copied and
                                         the call returns when the copy is done;
-                                        page-locked frames are pulled by one queued
-                                        kernel per batch over the host link */
+                                        page-locked frames are pulled over the host
+                                        link by queued kernels: those of the batch's
+                                        first front-end launch before it, the others'
+                                        by a few blocks of the launch before theirs */
 #define KF_FRAME_DEVICE 1            /* device memory of this device, read in place */
 #define KF_FRAME_HOST_COPY_ENGINE 2  /* host memory, moved by cudaMemcpyAsync on the
                                         batch's stream into a staging buffer of the

@@ -346,8 +346,9 @@ __global__ void __launch_bounds__(kTx* kTy, KF_FE_MINB) k_frontend_fused(DescLis
     }
   }
   __syncthreads();
-  // bilateral filter over the R0 x R0 region: w = 2^(sw2 - dz^2 c2), the
-  // k_bilateral weight with the exponent pre-scaled by log2(e)
+  // bilateral filter over the R0 x R0 region: w = 2^(sw2 - dz^2 c2), the weight
+  // exp(-(dx^2 + dy^2) / (2 sigma_s^2) - dz^2 / (2 sigma_r^2)) with its exponent
+  // scaled by log2(e)
 #if KF_FE_PAIRS
   // two vertically adjacent pixels per step (rows ly and ly + 1; a region
   // with an odd row count filters one row below it and drops the result)
@@ -372,7 +373,8 @@ __global__ void __launch_bounds__(kTx* kTy, KF_FE_MINB) k_frontend_fused(DescLis
   });
 #endif
   __syncthreads();
-  // pyramid: level l+1 from level l inside shared memory (same rule as k_downsample)
+  // pyramid: level l+1 from level l inside shared memory, the mean of the depths of
+  // a 2 x 2 block within 3 sigma_r of its first valid one
   float* lev[4] = {s_d0, s_d1, s_d2, s_d3};
 #pragma unroll
   for (int l = 0; l + 1 < KF_MAX_LEVELS; ++l) {

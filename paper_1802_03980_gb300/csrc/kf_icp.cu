@@ -13,7 +13,8 @@
 // of that window, associates again with the band known. Each stage's per-pair
 // epilogue (median and band after the histogram; solve and update after the
 // reduction) runs in the pair's last block to finish, found with a per-pair
-// arrival counter (no block ever waits for another).
+// arrival counter: no block waits for the others of its stage (the queue's blocks
+// wait for their next task only, each for a bounded time).
 #include "kf_icp.cuh"
 
 // Tuning of the ICP kernels: minimum resident blocks per SM (register cap).
@@ -29,8 +30,9 @@
 // Scheduled kernel: the pair's median epilogue also runs the reduction pass
 // of a hit while the pairs still running number at least the launch's
 // blocks / KF_FUSE_GRID_DIV (0: never; a large value: always). Measured at
-// 640x480 on 304 blocks: 256 pairs 4.60 ms never, 4.39 ms from 64 pairs on;
-// 64 pairs 1.45 ms never, 1.49 ms from 32 on.
+// 640x480 on 304 blocks: 256 pairs 3.40 ms never, 3.31 ms from 76 pairs on. Below,
+// spread over blocks for latency (with register gathers, before the ring: 64 pairs
+// 1.45 ms never, 1.49 ms from 32 on).
 #ifndef KF_FUSE_GRID_DIV
 #define KF_FUSE_GRID_DIV 4
 #endif
@@ -1208,7 +1210,7 @@ struct NoAllocArgs {
 // model pixels), which a pixel-by-pixel loop pays 16 times over. kShort: a model up to 2^22
 // pixels wide and high and no tiny bins (see project, bin_of).
 // Measured on GB300, 640x480: 28.4 us with a set-up launch, pixel by pixel and
-// a float64 chain over the items; 13.3 us now (calls in a row, the host's
+// a float64 chain over the items; 12.5 us now (calls in a row, the host's
 // part included).
 constexpr int kNoAllocFly = 8;
 template <bool kShort>

@@ -40,7 +40,8 @@
 // the time-out status that the host wrote before the launch.
 //
 // Measured on GB300, set frame and align of one pair, queue -> team: 160x120
-// (one level) 189 -> 107 us, 640x480 341 -> 179 us, 1280x960 ~490 -> 299 us.
+// (one level) 189 -> 100 us, 640x480 302 -> 158 us, 1280x960 430 -> 272 us (more
+// sizes and batches at kTeamSlots).
 #include "kf_icp.cuh"
 
 namespace kf {

@@ -210,8 +210,9 @@ __global__ void __launch_bounds__(256) k_cull_bricks(VolGeom g, Xf12 xf, Frustum
 // observed value <= 0 marks itself and its neighbours in `near` (and their
 // superbricks), where the raycast has to look; marks are never taken back
 // (until a reset).
-// Measured on GB300, 512^3 and 640x480, a whole call: 214 us with a thread per
-// voxel of every brick in the image, 69 us now.
+// Measured on GB300, 512^3 and 640x480, a whole call by events, calls in a row: 214
+// us with a thread per voxel of every brick in the image, 57 to 70 us now (four
+// scenes).
 template <bool kAny>
 __global__ void __launch_bounds__(256) k_integrate_bricks(float2* FW, VolGeom g, const float* D, Cam32 cam,
                                                           Xf12 xf, int nb, const int* list,
@@ -367,8 +368,8 @@ struct RayParams {
 // positive one ends it).
 // What bounds it is latency and issue per sample; a 640x480 view of a room takes
 // about 115 samples a ray to the surface, of which this looks up a dozen.
-// Measured on GB300, 512^3 and 640x480: 587 us looking up every sample, 88 us
-// now.
+// Measured on GB300, 512^3 and 640x480, calls in a row: 587 us looking up every
+// sample, 78 to 88 us now (four scenes).
 template <bool kAny>
 __global__ void __launch_bounds__(128) k_raycast(const float2* FW, VolGeom g, NearMap near, Cam32 cam,
                                                  RayParams rp, float* V, float* N) {
@@ -447,8 +448,9 @@ __global__ void __launch_bounds__(128) k_raycast(const float2* FW, VolGeom g, Ne
     ++k;
   }
   // the normals' samples once for all rays of the warp, wherever each met its
-  // surface: inside the loop they ran for each sample at which some ray met it (map
-  // and raycast at 512^3 and 640x480: 100 -> 96 us)
+  // surface: inside the loop they ran for each sample at which some ray met it
+  // (integration and raycast at 512^3 and 640x480, three volumes on three streams in
+  // turn: 100 -> 96 us a pass)
   __syncwarp();
   if (hit) {
     const float zs = __fadd_rn(zp, __fmul_rn(rp.dz, __fdiv_rn(fp, __fsub_rn(fp, fh))));
